@@ -74,6 +74,7 @@ struct GemmParams {
   float* splitk_ws;     // optional fp32 workspace for split tiles (NULL: whole tiles only)
   size_t splitk_ws_elems;
   int* splitk_flags;    // kMaxGemmCtas * 4 ints, zero before the first launch
+  int w_const;          // fp32: no kernel writes W, so it may be read before the previous kernel ends
   int* launches;        // optional host counter: kernels launched are added to it
   float* vnorm_out;     // kEpiRope: if set, ||v|| of each row's value heads, [M, (N - rope_cols) / hd]
 };
@@ -137,9 +138,12 @@ bool swap_preferred(int epi, int M, int N, int K);
 cudaError_t launch_gemm_swap(const void* A, int lda, const TcWeights& W, int epi,
                              const GemmParams& p, cudaStream_t s);
 
-// fp32 CUDA-core GEMM, same epilogues (kEpiRope is applied by launch_rope_f32).
-cudaError_t launch_gemm_f32(const float* A, int lda, const float* W, const float* W2, int epi,
-                            const GemmParams& p, cudaStream_t s);
+// fp32 CUDA-core GEMM, same epilogues; kEpiRope for head sizes that
+// gemm_f32_rope_supported names (powers of two from 8 to 128), with heads on
+// whole multiples of hd (otherwise store, then launch_rope_f32).
+bool gemm_f32_rope_supported(int hd);
+cudaError_t launch_gemm_f32(const float* A, int lda, const TcWeights& W, int epi, const GemmParams& p,
+                            cudaStream_t s);
 
 // ---- attention (k_attn.cu)
 // Two-tile tcgen05 attention (k_attn_pp.cu) for bf16 heads of 64 or 128 dims,

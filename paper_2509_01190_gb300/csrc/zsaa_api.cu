@@ -495,9 +495,8 @@ zsaa_status linear(zsaa_model* m, const void* A, int lda, const TcWeights& W, in
   if (m->cfg.dtype == ZSAA_BF16) {
     ZCK(launch_gemm_tc(A, lda, W, epi, p, s));
   } else {
-    if (epi == kEpiRope) return fail(ZSAA_ERR_UNSUPPORTED, "f32 RoPE epilogue");
-    ZCK(launch_gemm_f32(static_cast<const float*>(A), lda, static_cast<const float*>(W.w0),
-                        static_cast<const float*>(W.w1), epi, p, s));
+    p.w_const = 1;
+    ZCK(launch_gemm_f32(static_cast<const float*>(A), lda, W, epi, p, s));
   }
   return ZSAA_OK;
 }
@@ -590,14 +589,14 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
     p.K = d;
     p.out = m->qkv;
     p.ldo = m->ld_qkv;
-    if (dt == ZSAA_BF16) {
+    if (dt == ZSAA_BF16 || gemm_f32_rope_supported(hd)) {
       p.N = m->ld_qkv;
       p.pos = m->pos[cur];
       p.cos_t = m->rope_cos;
       p.sin_t = m->rope_sin;
       p.rope_cols = m->dq + m->dkv;
       p.hd = hd;
-      p.vnorm_out = m->vnorm;
+      if (dt == ZSAA_BF16) p.vnorm_out = m->vnorm;  // the fp32 column mass computes the norms itself
       TcWeights W{LW(m, li, kWq), LW(m, li, kWk), LW(m, li, kWv), m->dq, m->dq + m->dkv};
       TRACE("gemm_qkv_rope", 2.0 * Md * m->ld_qkv * d, (Md * d + static_cast<double>(m->ld_qkv) * d + Md * m->ld_qkv) * es);
       trace_scope_.kernels = 0;
@@ -1860,8 +1859,7 @@ zsaa_status zsaa_op_linear(const void* A, const void* W, const void* W2, const v
     ZCK(launch_gemm_tc(A, K, Wt, epilogue, p, s));
   } else if (dtype == ZSAA_F32) {
     if (epilogue == kEpiRope) return fail(ZSAA_ERR_UNSUPPORTED, "f32 GEMM has no RoPE epilogue");
-    ZCK(launch_gemm_f32(static_cast<const float*>(A), K, static_cast<const float*>(W),
-                        static_cast<const float*>(W2), epilogue, p, s));
+    ZCK(launch_gemm_f32(static_cast<const float*>(A), K, TcWeights{W, W2, nullptr, N, N}, epilogue, p, s));
   } else {
     return fail(ZSAA_ERR_INVALID_ARG, "bad dtype");
   }

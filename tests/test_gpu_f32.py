@@ -1,0 +1,55 @@
+"""The float32 kernels at the sizes where their tiling can go wrong: GEMM tiles
+of 64 x 64 x 16 with K split over clusters."""
+
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import zsaa_oracle as O
+from paper_2509_01190_gb300 import inputs as I
+from tests.helpers import accum_bound, need_gpu
+from tests.test_gpu_forward import check_case, run_case
+from tests.test_gpu_ops import _np, _rand
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def z(zlib):
+    need_gpu()
+    return zlib
+
+
+# K below one stage, off the 16-byte copies (70, 5), split over 2..8 CTAs of a
+# cluster (few tiles, deep K) and whole (many tiles); ragged rows and columns.
+@pytest.mark.parametrize("M,N,K", [(1, 3, 5), (64, 64, 16), (65, 130, 70), (63, 65, 15), (129, 96, 272),
+                                   (20, 200, 1027), (64, 128, 4096), (300, 516, 512), (1500, 1028, 100)])
+@pytest.mark.parametrize("epi", ["store", "resid", "swiglu"])
+def test_linear_f32_tiles(z, epi, M, N, K):
+    A, W, W2 = (_rand(s, i, dtype=torch.float32) for i, s in enumerate([(M, K), (N, K), (N, K)]))
+    H = _rand((M, N), 3, dtype=torch.float32)
+    h0 = _np(H)
+    e = {"store": z.EPI_STORE, "resid": z.EPI_RESID, "swiglu": z.EPI_SWIGLU}[epi]
+    out = H if epi == "resid" else torch.full((M, N), float("nan"), device="cuda")
+    z.zsaa_op_linear(A, W, W2 if epi == "swiglu" else None, H if epi == "resid" else None, out, M, N, K,
+                     z.ZSAA_F32, e)
+    torch.cuda.synchronize()
+    acc, u = _np(A) @ _np(W).T, _np(A) @ _np(W2).T
+    ref = {"store": acc, "resid": h0 + acc, "swiglu": O.silu(acc) * u}[epi]
+    b = accum_bound(_np(A), _np(W))
+    tol = {"store": b, "resid": b, "swiglu": 1.1 * np.abs(u) * b
+           + np.abs(O.silu(acc)) * accum_bound(_np(A), _np(W2))}[epi]
+    # plus the rounding of the epilogue's own few operations
+    assert np.all(np.abs(_np(out) - ref) <= tol + 5e-7 * np.abs(ref))
+
+
+# The QKV projection's fused RoPE for each way a head lies in a 64-column tile
+# (hd 16, 64 and 128, odd head counts), and the separate kernel's (hd 48).
+@pytest.mark.parametrize("d,heads,kv,hd,L", [(96, 3, 1, 16, 33), (256, 3, 1, 64, 70), (128, 2, 1, 128, 65),
+                                             (192, 4, 2, 48, 40), (512, 8, 8, 64, 130)])
+def test_forward_f32_head_sizes(z, d, heads, kv, hd, L):
+    shape = dataclasses.replace(I.TINY_F32, name="f32-heads", d_model=d, n_heads=heads, n_kv_heads=kv, head_dim=hd,
+                                ffn_dim=200, vocab=333)
+    check_case(run_case(z, shape, 2, L, 2.0, seqs=[0, 1]), "f32")
