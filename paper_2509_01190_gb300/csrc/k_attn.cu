@@ -16,7 +16,8 @@
 // enter P V as a hi/lo pair of bf16 matrices.  The column-mass
 // pass sweeps key blocks outer / query blocks inner so each CTA owns its
 // columns and sums them in registers (deterministic, no atomics).
-// fp32 path: plain CUDA-core kernels (one warp per row / column).
+// fp32 path: CUDA-core kernels, tiled (k_attn_f32.cu) for heads of 32, 64 or
+// 128 dims, one warp per row / column below for the others.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -479,6 +480,9 @@ cudaError_t launch_attention(int dtype, const void* qkv, int B, int N, int Hq, i
                              const uint8_t* key_alive) {
   if ((cu != nullptr || key_alive != nullptr) && dtype != ZSAA_BF16) return cudaErrorInvalidValue;
   const float scale_log2 = kLog2e / sqrtf(static_cast<float>(hd));
+  if (dtype == ZSAA_F32 && attention_f32_tiled(qkv, hd))
+    return launch_attention_f32_tiled(static_cast<const float*>(qkv), B, N, Hq, Hkv, hd, static_cast<float*>(out),
+                                      lse, scale_log2, causal, s);
   if (dtype == ZSAA_F32) {
     dim3 grid((N + 3) / 4, Hq, B);
     ZSAA_LAUNCH(attn_fwd_f32_kernel, dim3(grid), dim3(128), 0, s, static_cast<const float*>(qkv), N, Hq, Hkv, hd,
@@ -528,6 +532,9 @@ cudaError_t colmass_parts(int dtype, const void* qkv, const float* lse, const fl
                              status, n_qc, causal, s, cu, rows, q_alive);
   if (cu != nullptr || q_alive != nullptr) return cudaErrorInvalidValue;  // tensor-core path only
   const float scale_log2 = kLog2e / sqrtf(static_cast<float>(hd));
+  if (dtype == ZSAA_F32 && attention_f32_tiled(qkv, hd))
+    return launch_colmass_f32_tiled(static_cast<const float*>(qkv), lse, B, N, Hq, Hkv, hd, weight_vnorm, parts,
+                                    n_qc, scale_log2, causal, s);
   if (dtype == ZSAA_F32) {
     *n_qc = 1;
     dim3 grid((N + 3) / 4, Hkv, B);

@@ -175,6 +175,15 @@ cudaError_t launch_attention(int dtype, const void* qkv, int B, int N, int Hq, i
                              const int* cu = nullptr, const uint8_t* key_alive = nullptr);
 // key_alive (bf16, fixed length): [B, N] flags of the masked mode; keys with 0
 // are hidden from every query.
+// fp32 tiled kernels (k_attn_f32.cu): heads of 32, 64 or 128 dims, 16-byte
+// aligned qkv.  launch_attention and the column-mass launchers take them where
+// attention_f32_tiled says so, and one warp per row for the other head sizes.
+bool attention_f32_tiled(const void* qkv, int hd);
+cudaError_t launch_attention_f32_tiled(const float* qkv, int B, int N, int Hq, int Hkv, int hd, float* out,
+                                       float* lse, float scale_log2, int causal, cudaStream_t s);
+cudaError_t launch_colmass_f32_tiled(const float* qkv, const float* lse, int B, int N, int Hq, int Hkv, int hd,
+                                     int weight_vnorm, float* parts, int* n_chunks, float scale_log2, int causal,
+                                     cudaStream_t s);
 // Column mass C[B, Hkv, N] (via partial sums in `parts`, which must hold
 // colmass_parts_elems(B, N, Hq, Hkv) floats).  bf16 with a status word runs
 // the tensor-core kernel (k_colmass_tc.cu); otherwise the mma.sync / fp32 ones.

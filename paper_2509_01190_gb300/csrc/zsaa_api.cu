@@ -675,7 +675,7 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
         float* sc = want_scores ? opts->scores_out + off_scores : m->scores;
         const double pairs = static_cast<double>(B) * Hq * n_pairs(N);
         const int32_t* idx = m->idx;
-        if (dt == ZSAA_BF16 && !forced && k < N && N <= kSelectPartsMaxN) {
+        if (!forced && k < N && N <= kSelectPartsMaxN) {
           // column-mass partials, then top-k with the score reduction fused in
           int n_qc = 1;
           {

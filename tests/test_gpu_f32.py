@@ -1,5 +1,6 @@
 """The float32 kernels at the sizes where their tiling can go wrong: GEMM tiles
-of 64 x 64 x 16 with K split over clusters."""
+of 64 x 64 x 16 with K split over clusters, attention and column-mass tiles of
+16, 32 or 64 rows by 64 columns."""
 
 import dataclasses
 
@@ -11,7 +12,7 @@ from oracle import zsaa_oracle as O
 from paper_2509_01190_gb300 import inputs as I
 from tests.helpers import accum_bound, need_gpu
 from tests.test_gpu_forward import check_case, run_case
-from tests.test_gpu_ops import _np, _rand
+from tests.test_gpu_ops import _np, _oracle_attention, _qkv, _rand
 
 pytestmark = pytest.mark.gpu
 
@@ -43,6 +44,28 @@ def test_linear_f32_tiles(z, epi, M, N, K):
            + np.abs(O.silu(acc)) * accum_bound(_np(A), _np(W2))}[epi]
     # plus the rounding of the epilogue's own few operations
     assert np.all(np.abs(_np(out) - ref) <= tol + 5e-7 * np.abs(ref))
+
+
+# Every head size of the tiled kernels and one of the row kernels (96), tile
+# edges, odd head ratios; the many-head cases take the 64-row tiles.
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("B,N,Hq,Hkv,hd", [(1, 1, 2, 2, 64), (2, 15, 3, 1, 128), (1, 17, 4, 2, 32), (2, 63, 4, 4, 64),
+                                           (1, 65, 2, 1, 128), (1, 130, 6, 2, 32), (4, 193, 24, 8, 64),
+                                           (4, 129, 32, 8, 32), (4, 257, 20, 4, 128), (1, 50, 2, 1, 96)])
+def test_attention_and_colmass_f32_tiles(z, B, N, Hq, Hkv, hd, causal):
+    qkv = _qkv(B, N, Hq, Hkv, hd, 90 + N, torch.float32)
+    out = torch.full((B * N, Hq * hd), float("nan"), device="cuda")
+    lse = torch.full((B, Hq, N), float("nan"), device="cuda")
+    C = torch.full((B, Hkv, N), float("nan"), device="cuda")
+    z.zsaa_op_attention_ex(qkv, B, N, Hq, Hkv, hd, z.ZSAA_F32, causal, out, lse)
+    z.zsaa_op_colmass_ex(qkv, lse, B, N, Hq, Hkv, hd, z.ZSAA_F32, causal, C)
+    torch.cuda.synchronize()
+    ref_o, ref_lse, Ps, _ = _oracle_attention(qkv, B, N, Hq, Hkv, hd, causal=causal)
+    # the bounds of the float32 checks in test_gpu_ops.py
+    np.testing.assert_allclose(_np(out).reshape(B, N, Hq * hd), ref_o, rtol=1e-5, atol=1e-5)
+    np.testing.assert_allclose(_np(lse), ref_lse, rtol=1e-5, atol=1e-4)
+    refC = np.stack([O.column_mass(Ps[b], Hkv) for b in range(B)])
+    np.testing.assert_allclose(_np(C), refC, rtol=1e-5, atol=1e-6)
 
 
 # The QKV projection's fused RoPE for each way a head lies in a 64-column tile
