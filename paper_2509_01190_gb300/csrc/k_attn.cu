@@ -516,7 +516,7 @@ int colmass_chunks(int N) {
 }
 
 size_t colmass_parts_elems(int B, int N, int Hq, int Hkv) {
-  const int tc_chunks = 2 * (Hq / Hkv);  // the tensor-core kernel: (head, column half)
+  const int tc_chunks = 2 * (Hq / Hkv);  // the tensor-core kernel: (head, half of its queries)
   const int c = colmass_chunks(N) > tc_chunks ? colmass_chunks(N) : tc_chunks;
   return static_cast<size_t>(c) * B * Hkv * N;
 }

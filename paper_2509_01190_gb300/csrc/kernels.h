@@ -208,8 +208,9 @@ cudaError_t launch_position_parts(int dtype, const void* qkv, const float* lse, 
                                   int* n_qc, int* status, int causal, cudaStream_t s,
                                   const int* cu = nullptr, int rows = 0,
                                   const uint8_t* q_alive = nullptr);
-// Tensor-core column-mass partials: parts[Hq/Hkv][B][Hkv][N] (per head of the
-// group), times vnorm when it is not NULL; hd 64 or 128.  With cu: packed
+// Tensor-core column-mass partials: parts[chunks][B][Hkv][N] (a chunk per head of
+// the group, or two per head for the halves of its queries; *n_chunks of them),
+// times vnorm when it is not NULL; hd 64 or 128.  With cu: packed
 // sequences of different lengths (rows [cu[b], cu[b+1]), `rows` in all, N the
 // longest); vnorm is then per packed row.
 cudaError_t launch_colmass_tc(const void* qkv, const float* lse, const float* vnorm, int B, int N,
