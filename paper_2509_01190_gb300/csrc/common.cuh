@@ -93,6 +93,25 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
   return t;
 }
 
+// n / d for 0 <= n < 2^31, d >= 1 (a work item's index is decoded by every role
+// of a persistent kernel; a plain division is a long dependent chain)
+struct FastDiv {
+  int d;
+  uint32_t m;  // about 2^32 / d
+  __device__ __forceinline__ int div(int n, int& rem) const {
+    int q = static_cast<int>(__umulhi(static_cast<uint32_t>(n), m));
+    rem = n - q * d;  // m is 2^32 / d rounded down: q is at most one short
+    if (rem >= d) {
+      ++q;
+      rem -= d;
+    }
+    return q;
+  }
+};
+inline FastDiv fast_div(int d) {
+  return FastDiv{d, d == 1 ? 0xffffffffu : static_cast<uint32_t>((1ull << 32) / static_cast<uint32_t>(d))};
+}
+
 // Variable-length batches keep the rows of B sequences packed, sequence b at
 // rows [cu[b], cu[b+1]) (cu[0] = 0, strictly increasing).  Sequence of row r:
 __device__ __forceinline__ int seq_of_row(const int* __restrict__ cu, int B, int r) {

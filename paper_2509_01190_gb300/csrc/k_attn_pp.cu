@@ -2,9 +2,11 @@
 // tensor cores: two query tiles per CTA whose softmaxes take turns, so each
 // tile's exponentials run while the tensor core works on the other tile.
 //
-// A work item is (sequence b, KV group g, pair of query heads h0 and h0+1 of
-// that group, block of 128 queries).  Both heads read the same keys and
-// values, so each K/V block is loaded once for the two tiles.  Per key block
+// A work item is two tiles of 128 queries that read the same keys and values,
+// so each K/V block is loaded once for both: two query heads of a KV group
+// (an even number of heads per group), or two neighbouring query blocks of one
+// head (an odd number; with the causal mask the first tile has fewer key
+// blocks, and the last block of a sequence may have no partner).  Per key block
 // j of 128 keys (causal: up to the diagonal):
 //   S_x = Q_x K_j^T                      (tcgen05, M = 128, N = 128, K = hd)
 //   softmax warps of tile x (one query row per thread, TMEM lane = row):
@@ -23,7 +25,21 @@
 // Tensor-core order (one issuing thread; tcgen05.mma executes in issue order):
 //   S_A(0) S_B(0) | PV_A(0) S_A(1) PV_B(0) S_B(1) | PV_A(1) S_A(2) PV_B(1) ...
 // so tile A's softmax of block j+1 runs under PV_B(j) and S_B(j+1), and tile
-// B's under PV_A(j+1) and S_A(j+2).
+// B's under PV_A(j+1) and S_A(j+2).  An item's last P V is followed by the next
+// item's first S in the same way, and its epilogue runs under the next item's
+// first P V (with heads of 64 dims O has two buffers per tile for that).
+//
+// What bounds it: on long sequences the MMA stream (24 MMAs per tile and key
+// block, 16 of them P V), on short ones the chain softmax -> P V -> epilogue of
+// an item and the fetches of code that runs only once or twice per CTA.  So 32-
+// column chunks with no visible key are skipped (only their P is zeroed), MMAs
+// cover the live keys alone, and the code has one copy of each part: two copies
+// of the conversion (an unrolled pair of chunks, or masked and unmasked) cost
+// 5-25% at one or two key blocks.  Measured before and after (causal, 32 heads
+// over 8 groups): 4 x 2048 rows of 128 dims 201 -> 185 us, 64 x 256 of 64 dims
+// 84 -> 77, 64 x 30 34 -> 25; 16 x 501, 16 heads without groups, no mask: 75
+// (one tile per CTA and a transposed V) -> 52; 1 x 2048, 32 such heads of 128
+// dims, causal: 121 -> 55.
 //
 // Roles (384 threads): warp 0 TMA producer (both Q tiles per item; K and V of
 // every key block through a ring), warp 1 MMA issuer, warps 4-7 tile A's
@@ -48,53 +64,84 @@ struct PpCfg {
   static constexpr int CH = HD / 64;                 // 64-dim (128-byte) chunks
   static constexpr int TILE = PP_BM * HD * 2;        // one Q tile, K block or V block
   static constexpr int STAGES = HD == 128 ? 2 : 4;   // K/V ring
+  static constexpr int O_BUFS = 128 / HD;            // O accumulators per tile
   static constexpr size_t SMEM = 2 * static_cast<size_t>(TILE) + 2 * STAGES * static_cast<size_t>(TILE) + 256 + 1024;
 };
 static_assert(PpCfg<64>::SMEM <= 227 * 1024 && PpCfg<128>::SMEM <= 227 * 1024, "shared memory");
 
 __host__ __device__ constexpr uint32_t s_col(int x) { return 256u * x; }
-__host__ __device__ constexpr uint32_t o_col(int x) { return 256u * x + 128u; }
+template <int HD>
+__host__ __device__ constexpr uint32_t o_col(int x, uint32_t buf) {
+  return 256u * x + 128u + HD * buf;
+}
 
 struct PpArgs {
   float* lse2;  // [B, Hq, N], log2 domain
-  bf16* out;    // [B*N, Hq*hd]
-  int B, N, Hq, Hkv, pairs, n_qb, causal;
+  bf16* out;    // [B*N (or the packed rows), Hq*hd]
+  int B, N, Hq, Hkv, n_qb, causal, total;
+  int by_head;   // 1: the two tiles are neighbouring heads, 0: neighbouring query blocks of one head
+  int wide_out;  // out allows 32-byte stores
+  FastDiv inner, units, groups;  // items per query position, heads (or pairs) per group, groups
+  const int* cu;  // packed sequences of different lengths: rows [cu[b], cu[b+1]); N = the longest
   float scale_log2;
   int* status;
 };
 
 struct PpItem {
-  int qb, b, g, h0, n_kb;
+  int b, g, row0, n;         // sequence, KV group, first row and length of the sequence
+  int h[2], qb[2], nk[2];    // per tile: head, query block, key blocks (0: no such tile)
+  int n_kb;                  // key blocks of the item
 };
 
-// The r-th work item of this CTA: items are numbered longest query blocks
-// first and dealt to the CTAs in a snake order (0..G-1, then G-1..0, ...), so
-// the causal triangle's long and short items even out across CTAs.  Returns
-// an index >= total once the CTA has none left (the sequence only grows).
-__device__ __forceinline__ int pp_item_index(int r) {
-  const int G = gridDim.x, i = blockIdx.x;
-  return r * G + ((r & 1) ? G - 1 - i : i);
+// Work item t, longest query blocks first; false when its sequence has no such queries.
+__device__ __forceinline__ bool pp_item(int t, const PpArgs& a, PpItem& it) {
+  int r, u;
+  const int qp = (a.by_head ? a.n_qb : (a.n_qb + 1) / 2) - 1 - a.inner.div(t, r);
+  r = a.units.div(r, u);
+  it.b = a.groups.div(r, it.g);
+  if (a.cu) {
+    it.row0 = a.cu[it.b];
+    it.n = a.cu[it.b + 1] - it.row0;
+  } else {
+    it.row0 = it.b * a.N;
+    it.n = a.N;
+  }
+  const int h0 = it.g * (a.by_head ? 2 * a.units.d : a.units.d) + (a.by_head ? 2 * u : u);
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    it.h[x] = a.by_head ? h0 + x : h0;
+    it.qb[x] = a.by_head ? qp : 2 * qp + x;
+    const int keys = a.causal ? min(it.n, (it.qb[x] + 1) * PP_BM) : it.n;
+    it.nk[x] = it.qb[x] * PP_BM < it.n ? (keys + PP_BN - 1) / PP_BN : 0;
+  }
+  it.n_kb = max(it.nk[0], it.nk[1]);
+  return it.nk[0] > 0;  // tile 0's queries come first
 }
 
-// Work item t, longest query blocks first.
-__device__ __forceinline__ PpItem pp_item(int t, const PpArgs& a) {
-  PpItem it;
-  const int per_qb = a.B * a.Hkv * a.pairs;
-  it.qb = a.n_qb - 1 - t / per_qb;
-  int r = t % per_qb;
-  const int hp = r % a.pairs;
-  r /= a.pairs;
-  it.g = r % a.Hkv;
-  it.b = r / a.Hkv;
-  it.h0 = it.g * (a.Hq / a.Hkv) + 2 * hp;
-  const int keys = a.causal ? min(a.N, (it.qb + 1) * PP_BM) : a.N;
-  it.n_kb = (keys + PP_BN - 1) / PP_BN;
-  return it;
+// This CTA's items: numbered longest query blocks first and dealt to the CTAs
+// in a snake order (0..G-1, then G-1..0, ...), so the causal triangle's long
+// and short items even out across CTAs.  Advances r to the next live item;
+// false once there is none.
+__device__ __forceinline__ bool pp_next(int& r, const PpArgs& a, PpItem& it) {
+  const int G = gridDim.x, i = blockIdx.x;
+  while (true) {
+    if (r * G >= a.total) return false;
+    const int t = r * G + ((r & 1) ? G - 1 - i : i);
+    ++r;
+    if (t < a.total && pp_item(t, a, it)) return true;
+  }
 }
 
 __device__ __forceinline__ float ex2_fast(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// max of three in one instruction (the rate of a two-operand maximum)
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
   return y;
 }
 
@@ -124,6 +171,13 @@ __device__ __forceinline__ void tc_mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem,
       : "memory");
 }
 
+// 32 bytes to a 32-byte aligned address.
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* w) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+               "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+
 // Warp-collective: lane i writes TMEM lane (base + i), 32 consecutive columns.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   tmem_st16(taddr, *reinterpret_cast<const uint32_t(*)[16]>(r));
@@ -131,11 +185,46 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 }
 
 
+// The two products of a key block, issued by one thread.  Not inlined: a CTA
+// with one or two short items runs this code cold, and its instruction fetches
+// are then a good part of its time.
+template <int HD>
+__device__ __noinline__ void pp_issue_s(uint32_t qa, uint32_t ka, uint32_t d_tmem, int keys, uint64_t* done) {
+  const uint32_t idesc = idesc_bf16_f32(PP_BM, (keys + 15) & ~15);  // the block's live keys
+#pragma unroll
+  for (int kk = 0; kk < HD / 16; ++kk)
+    tc_mma_bf16(d_tmem, sdesc_sw128(qa + (kk / 4) * (PP_BM * 128) + (kk % 4) * 32),
+                sdesc_sw128(ka + (kk / 4) * (PP_BN * 128) + (kk % 4) * 32), idesc, kk > 0 ? 1u : 0u);
+  tc_commit(done);
+}
+// O (+)= P_hi V + P_lo V over the 16-key steps that hold a key.
+template <int HD>
+__device__ __noinline__ void pp_issue_pv(uint32_t va, uint32_t p_tmem, uint32_t o_tmem, bool first, int keys) {
+  constexpr uint32_t idesc = idesc_bf16_f32(PP_BM, HD) | (1u << 16);  // B (V) MN-major
+  // V's 64-dim chunks are PP_BN * 128 bytes apart; with one chunk (hd 64) the
+  // stride is never used and is set to the 8-row atom stride, so the
+  // descriptor addresses only the 16 keys of each MMA either way.
+  constexpr uint32_t kVChunkStride = HD > 64 ? PP_BN * 128 : 1024;
+  auto mma = [&](int part, int kk) {
+    tc_mma_bf16_ts(o_tmem, p_tmem + 32 * (kk / 2) + 16 * part + 8 * (kk % 2),
+                   sdesc_sw128_mn(va + kk * 16 * 128, kVChunkStride), idesc, (first && part == 0 && kk == 0) ? 0u : 1u);
+  };
+  if (keys == PP_BN) {  // (no test between the issues: they bound the long sequences)
+#pragma unroll
+    for (int part = 0; part < 2; ++part)
+#pragma unroll
+      for (int kk = 0; kk < PP_BN / 16; ++kk) mma(part, kk);
+  } else {
+#pragma unroll 2
+    for (int i = 0; i < 2 * ((keys + 15) / 16); ++i) mma(i & 1, i >> 1);
+  }
+}
+
 template <int HD>
 __global__ void __launch_bounds__(PP_THREADS, 1)
     attn_pp_kernel(const __grid_constant__ CUtensorMap tm, const PpArgs a) {
   using C = PpCfg<HD>;
-  constexpr int CH = C::CH, TILE = C::TILE, ST = C::STAGES;
+  constexpr int CH = C::CH, TILE = C::TILE, ST = C::STAGES, NB = C::O_BUFS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -147,16 +236,15 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
   uint64_t* q_empty = bars + 1;         // [1]
   uint64_t* s_full = bars + 2;          // [2] per tile
   uint64_t* p_full = bars + 4;          // [2]
-  uint64_t* o_full = bars + 6;          // [2]
-  uint64_t* o_empty = bars + 8;         // [2]
-  uint64_t* mma_done = bars + 10;       // [1]
-  uint64_t* kv_full = bars + 11;        // [ST]
-  uint64_t* kv_empty = bars + 11 + ST;  // [ST]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 11 + 2 * ST);
+  uint64_t* o_full = bars + 6;          // [2][NB]
+  uint64_t* o_empty = bars + 10;        // [2][NB]
+  uint64_t* mma_done = bars + 14;       // [1]
+  uint64_t* kv_full = bars + 15;        // [ST]
+  uint64_t* kv_empty = bars + 15 + ST;  // [ST]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 15 + 2 * ST);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = a.n_qb * a.B * a.Hkv * a.pairs;
   pdl_trigger();
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -164,8 +252,10 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     for (int x = 0; x < 2; ++x) {
       mbar_init(&s_full[x], 1);
       mbar_init(&p_full[x], 4);
-      mbar_init(&o_full[x], 1);
-      mbar_init(&o_empty[x], 4);
+    }
+    for (int i = 0; i < 2 * NB; ++i) {
+      mbar_init(&o_full[i], 1);
+      mbar_init(&o_empty[i], 4);
     }
     mbar_init(mma_done, 1);
     for (int i = 0; i < ST; ++i) {
@@ -188,19 +278,19 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     if (lane == 0) {
       bool ok = true;
       uint32_t J = 0, items = 0, q_issued = 0;
-      for (int t = pp_item_index(0); t < total && ok; t = pp_item_index(++items)) {
-        const PpItem it = pp_item(t, a);
-        const int row0 = it.b * a.N;
+      PpItem it;
+      for (int r = 0; ok && pp_next(r, a, it); ++items) {
         if (!mbar_wait_ab(q_empty, (items & 1) ^ 1, a.status, abort_flag)) {
           ok = false;
           break;
         }
         ++q_issued;
-        mbar_arrive_expect_tx(q_full, 2 * TILE);
+        mbar_arrive_expect_tx(q_full, (it.nk[1] > 0 ? 2 : 1) * TILE);
         for (int x = 0; x < 2; ++x)
-          for (int c = 0; c < CH; ++c)
-            tma_load_2d(sQ + x * TILE + c * (PP_BM * 128), &tm, (it.h0 + x) * HD + c * 64,
-                        row0 + it.qb * PP_BM, q_full);
+          if (it.nk[x] > 0)
+            for (int c = 0; c < CH; ++c)
+              tma_load_2d(sQ + x * TILE + c * (PP_BM * 128), &tm, it.h[x] * HD + c * 64,
+                          it.row0 + it.qb[x] * PP_BM, q_full);
         for (int j = 0; j < it.n_kb; ++j, ++J) {
           const int st = J % ST;
           if (!mbar_wait_ab(&kv_empty[st], ((J / ST) & 1) ^ 1, a.status, abort_flag)) {
@@ -210,9 +300,9 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
           mbar_arrive_expect_tx(&kv_full[st], 2 * TILE);
           for (int c = 0; c < CH; ++c) {
             tma_load_2d(sK + st * TILE + c * (PP_BN * 128), &tm, (a.Hq + it.g) * HD + c * 64,
-                        row0 + j * PP_BN, &kv_full[st]);
+                        it.row0 + j * PP_BN, &kv_full[st]);
             tma_load_2d(sV + st * TILE + c * (PP_BN * 128), &tm, (a.Hq + a.Hkv + it.g) * HD + c * 64,
-                        row0 + j * PP_BN, &kv_full[st]);
+                        it.row0 + j * PP_BN, &kv_full[st]);
           }
         }
       }
@@ -226,82 +316,89 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(PP_BM, PP_BN);
-      constexpr uint32_t idesc_o = idesc_bf16_f32(PP_BM, HD) | (1u << 16);  // B (V) MN-major
-      // V's 64-dim chunks are PP_BN * 128 bytes apart; with one chunk (hd 64)
-      // the stride is never used and is set to the 8-row atom stride, so the
-      // descriptor addresses only the 16 keys of each MMA either way.
-      constexpr uint32_t kVChunkStride = CH > 1 ? PP_BN * 128 : 1024;
       bool ok = true;
-      uint32_t J = 0, items = 0;
-      auto issue_s = [&](int x, int st) {  // S_x = Q_x K^T
-        const uint32_t qa = smem_u32(sQ + x * TILE), ka = smem_u32(sK + st * TILE);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk)
-          tc_mma_bf16(tmem + s_col(x), sdesc_sw128(qa + (kk / 4) * (PP_BM * 128) + (kk % 4) * 32),
-                      sdesc_sw128(ka + (kk / 4) * (PP_BN * 128) + (kk % 4) * 32), idesc_s, kk > 0 ? 1u : 0u);
-        tc_commit(&s_full[x]);
+      uint32_t J = 0, items = 0;  // key blocks before this item, items begun
+      uint32_t n_p[2] = {0, 0}, n_o[2] = {0, 0};  // per tile: P blocks taken, items
+      auto issue_s = [&](int x, int st, int keys) {  // S_x = Q_x K^T over the block's `keys` live keys
+        pp_issue_s<HD>(smem_u32(sQ + x * TILE), smem_u32(sK + st * TILE), tmem + s_col(x), keys, &s_full[x]);
       };
-      auto issue_pv = [&](int x, int st, bool first) {  // O_x (+)= P_hi V + P_lo V
-        const uint32_t va = smem_u32(sV + st * TILE);
-#pragma unroll
-        for (int part = 0; part < 2; ++part)
-#pragma unroll
-          for (int kk = 0; kk < PP_BN / 16; ++kk)
-            tc_mma_bf16_ts(tmem + o_col(x), tmem + s_col(x) + 32 * (kk / 2) + 16 * part + 8 * (kk % 2),
-                           sdesc_sw128_mn(va + kk * 16 * 128, kVChunkStride), idesc_o,
-                           (first && part == 0 && kk == 0) ? 0u : 1u);
-      };
-      for (int t = pp_item_index(0); t < total && ok; t = pp_item_index(++items)) {
-        const PpItem it = pp_item(t, a);
-        if (!mbar_wait_ab(q_full, items & 1, a.status, abort_flag)) {
-          ok = false;
-          break;
+      // The S of an item's first block are issued under the item before it, each
+      // as soon as its tile's last P V is (s_left: S products of the item after
+      // this one not issued yet).
+      PpItem it, nx;
+      int r = 0;
+      bool have = pp_next(r, a, nx), begun = false;  // begun: nx's Q and first keys are there
+      int s_left = have ? nx.nk[0] + nx.nk[1] : 0;
+      auto first_s = [&](int x, uint32_t Jn) {
+        if (!begun) {
+          if (!mbar_wait_ab(q_full, items & 1, a.status, abort_flag) ||
+              !mbar_wait_ab(&kv_full[Jn % ST], (Jn / ST) & 1, a.status, abort_flag)) {
+            ok = false;
+            return;
+          }
+          tc_fence_after();
+          begun = true;
         }
+        issue_s(x, Jn % ST, min(PP_BN, nx.n));
+        if (--s_left == 0) tc_commit(q_empty);  // Q read for the last time
+      };
+      if (have) {
+        first_s(0, 0);
+        if (ok && nx.nk[1] > 0) first_s(1, 0);
+      }
+      while (have && ok) {
+        it = nx;
+        int left = s_left;  // this item's S products not issued yet
+        have = pp_next(r, a, nx);
+        s_left = have ? nx.nk[0] + nx.nk[1] : 0;
+        begun = false;
+        ++items;
+        bool early[2] = {false, false};  // the next item's first S issued
+        const uint32_t Jn = J + it.n_kb;
         for (int j = 0; j < it.n_kb && ok; ++j) {
           const uint32_t Jj = J + j;
-          const int st = Jj % ST;
-          if (j == 0) {
-            if (!mbar_wait_ab(&kv_full[st], (Jj / ST) & 1, a.status, abort_flag)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            issue_s(0, st);
-            issue_s(1, st);
-            if (it.n_kb == 1) tc_commit(q_empty);
-          }
-          const bool more = j + 1 < it.n_kb;
-          const int st1 = (Jj + 1) % ST;
+          const int st = Jj % ST, st1 = (Jj + 1) % ST;
+          const int keys = min(PP_BN, it.n - j * PP_BN);
+          bool next_kv = false;  // K_{j+1} waited for
           for (int x = 0; x < 2 && ok; ++x) {
-            // the epilogue of the previous item has read O_x out
-            if (j == 0 && items > 0 && !mbar_wait_ab(&o_empty[x], (items - 1) & 1, a.status, abort_flag)) {
+            if (j >= it.nk[x]) continue;
+            const uint32_t buf = n_o[x] % NB;
+            // the epilogue of the item that used this O last has read it out
+            if ((j == 0 && n_o[x] >= NB &&
+                 !mbar_wait_ab(&o_empty[x * NB + buf], (n_o[x] / NB - 1) & 1, a.status, abort_flag)) ||
+                !mbar_wait_ab(&p_full[x], n_p[x] & 1, a.status, abort_flag)) {
               ok = false;
               break;
             }
-            if (!mbar_wait_ab(&p_full[x], Jj & 1, a.status, abort_flag)) {
-              ok = false;
-              break;
-            }
+            ++n_p[x];
             tc_fence_after();
-            issue_pv(x, st, j == 0);
-            if (x == 1) tc_commit(&kv_empty[st]);  // K_j and V_j read for the last time
-            if (more) {
-              if (x == 0) {
+            pp_issue_pv<HD>(smem_u32(sV + st * TILE), tmem + s_col(x), tmem + o_col<HD>(x, buf), j == 0, keys);
+            if (x == 1 || j >= it.nk[1]) tc_commit(&kv_empty[st]);  // K_j and V_j read for the last time
+            if (j + 1 < it.nk[x]) {
+              if (!next_kv) {
                 if (!mbar_wait_ab(&kv_full[st1], ((Jj + 1) / ST) & 1, a.status, abort_flag)) {
                   ok = false;
                   break;
                 }
                 tc_fence_after();
+                next_kv = true;
               }
-              issue_s(x, st1);
-              if (x == 1 && j + 2 == it.n_kb) tc_commit(q_empty);  // Q read for the last time
+              issue_s(x, st1, min(PP_BN, it.n - (j + 1) * PP_BN));
+              if (--left == 0) tc_commit(q_empty);
             } else {
-              tc_commit(&o_full[x]);
+              tc_commit(&o_full[x * NB + buf]);
+              ++n_o[x];
+              // (while this item's S are outstanding its Q buffers are, too)
+              if (have && nx.nk[x] > 0 && left == 0) {
+                first_s(x, Jn);
+                early[x] = true;
+              }
             }
           }
         }
-        J += it.n_kb;
+        for (int x = 0; x < 2 && ok && have; ++x)
+          if (nx.nk[x] > 0 && !early[x]) first_s(x, Jn);
+        J = Jn;
       }
       // every MMA issued has finished before the CTA frees TMEM
       tc_commit(mma_done);
@@ -312,147 +409,214 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     // ---------------------------------------------------------------- softmax + epilogue
     const int x = (warp - 4) / 4;  // tile
     const int quad = warp & 3;
-    const int row = quad * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     const uint32_t s_addr = tmem + lane_off + s_col(x);
-    const uint32_t o_addr = tmem + lane_off + o_col(x);
     bool ok = true;
-    uint32_t J = 0, items = 0;
+    uint32_t J = 0;                      // key blocks of the items before this one
+    uint32_t n_s = 0, n_o = 0, n_e = 0;  // S blocks taken, items begun, epilogues done
     auto arrive = [&](uint64_t* bar) {
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
     };
-    for (int t = pp_item_index(0); t < total; t = pp_item_index(++items)) {
-      const PpItem it = pp_item(t, a);
-      const int q = it.qb * PP_BM + row;
-      float m = -INFINITY, l = 0.f;
-      for (int j = 0; j < it.n_kb; ++j) {
-        const uint32_t Jj = J + j;
-        ok = ok && __all_sync(0xffffffffu, mbar_wait_ab(&s_full[x], Jj & 1, a.status, abort_flag));
-        tc_fence_after();
-        // keys k0 + e with e >= lim are hidden (causal diagonal, sequence end)
-        const int k0 = j * PP_BN;
-        int lim = min(PP_BN, a.N - k0);
-        if (a.causal) lim = min(lim, q - k0 + 1);
-        if (ok) {
-          // masking (causal diagonal or sequence end) only where some lane of
-          // the warp needs it, so full blocks take the branch-free path
-          const bool masked = __any_sync(0xffffffffu, lim < PP_BN);
-          // pass 1: the block's row maximum, 64 columns per TMEM round trip
-          float mx = -INFINITY;
-#pragma unroll 1
-          for (int c = 0; c < PP_BN / 32; c += 2) {
-            uint32_t r[64];
-            tmem_ld32(s_addr + 32 * c, *reinterpret_cast<uint32_t(*)[32]>(r));
-            tmem_ld32(s_addr + 32 * c + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
-            tmem_ld_wait();
-            if (!masked) {
-#pragma unroll
-              for (int e = 0; e < 64; ++e) mx = fmaxf(mx, __uint_as_float(r[e]));
-            } else {
-#pragma unroll
-              for (int e = 0; e < 64; ++e)
-                if (32 * c + e < lim) mx = fmaxf(mx, __uint_as_float(r[e]));
-            }
-          }
-          const float mb = mx == -INFINITY ? -INFINITY : mx * a.scale_log2;
-          const bool need = mb > m + PP_RESCALE_LOG2;
-          if (__any_sync(0xffffffffu, need)) {
-            const float mn = need ? mb : m;
-            const float f = need ? (m == -INFINITY ? 0.f : exp2f(m - mn)) : 1.f;
-            if (j > 0) {  // O holds blocks 0..j-1 (PV_x(j-1) finished before S_x(j) was signalled)
-#pragma unroll 1
-              for (int c = 0; c < HD / 32; ++c) {
-                uint32_t r[32];
-                tmem_ld32(o_addr + 32 * c, r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * f);
-                tmem_st32(o_addr + 32 * c, r);
-              }
-            }
-            l *= f;
-            m = mn;
-          }
-          // pass 2: P as a bf16 pair over the S columns just read; the next
-          // chunk's load is in flight while this one is converted
-          // P = 2^(s*scale - m) split as hi = P rounded to bf16 and lo = P - hi
-          // (exact in fp32, then rounded to bf16), so hi + lo carries P to
-          // about 17 bits
-          const uint64_t scale2 = f2pack(a.scale_log2, a.scale_log2);
-          const uint64_t nm2 = f2pack(-m, -m);
-          auto emit = [&](const uint32_t (&r)[32], int c) {
-            uint32_t hi[16], lo[16];
-            uint64_t lsum = f2pack(0.f, 0.f);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              float t0, t1;
-              f2unpack(ffma2(f2pack(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), scale2, nm2), t0, t1);
-              float p0 = ex2_fast(t0), p1 = ex2_fast(t1);
-              if (masked) {
-                const int k = 32 * c + 2 * e;
-                p0 = k < lim ? p0 : 0.f;
-                p1 = k + 1 < lim ? p1 : 0.f;
-              }
-              const uint64_t pp = f2pack(p0, p1);
-              lsum = fadd2(lsum, pp);
-              hi[e] = pack_bf16x2(p0, p1);
-              float r0, r1;
-              f2unpack(fsub2(pp, f2pack(bf16lo(hi[e]), bf16hi(hi[e]))), r0, r1);
-              lo[e] = pack_bf16x2(r0, r1);
-            }
-            float l0, l1;
-            f2unpack(lsum, l0, l1);
-            l += l0 + l1;
-            tmem_st16(s_addr + 32 * c, hi);
-            tmem_st16(s_addr + 32 * c + 16, lo);
-          };
-          uint32_t ra[32], rb[32];
-          tmem_ld32(s_addr, ra);
-          tmem_ld_wait();
-#pragma unroll 1
-          for (int c = 0; c < PP_BN / 32; c += 2) {
-            tmem_ld32(s_addr + 32 * (c + 1), rb);
-            emit(ra, c);
-            tmem_ld_wait();
-            if (c + 2 < PP_BN / 32) tmem_ld32(s_addr + 32 * (c + 2), ra);
-            emit(rb, c + 1);
-            tmem_ld_wait();
-          }
-          tmem_st_wait();
-        }
-        tc_fence_before();
-        arrive(&p_full[x]);
-      }
-      J += it.n_kb;
-      // epilogue: O / l in bf16, and the row normaliser
-      ok = ok && __all_sync(0xffffffffu, mbar_wait_ab(&o_full[x], items & 1, a.status, abort_flag));
+    // the item whose epilogue is still to do: its row's output, normaliser and sums
+    bf16* e_out = nullptr;  // nullptr: the row is past the sequence's end
+    float* e_lse = nullptr;
+    float e_m = 0.f, e_l = 0.f;
+    // O / l in bf16, and the row normaliser
+    auto epilogue = [&]() {
+      const int buf = static_cast<int>(n_e % NB);
+      const uint32_t o_addr = tmem + lane_off + o_col<HD>(x, buf);
+      ok = ok && __all_sync(0xffffffffu, mbar_wait_ab(&o_full[x * NB + buf], (n_e / NB) & 1, a.status, abort_flag));
       tc_fence_after();
-      if (ok) {
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        const int h = it.h0 + x;
-        bf16* orow = a.out + (static_cast<size_t>(it.b) * a.N + q) * (static_cast<size_t>(a.Hq) * HD) + h * HD;
+      if (ok && __any_sync(0xffffffffu, e_out != nullptr)) {
+        const float inv = e_l > 0.f ? 1.f / e_l : 0.f;
 #pragma unroll 1
         for (int c = 0; c < HD / 32; ++c) {
           uint32_t r[32];
           tmem_ld32(o_addr + 32 * c, r);
           tmem_ld_wait();
-          if (q < a.N) {
+          if (e_out != nullptr) {
+            uint32_t w[16];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              uint4 w;
-              w.x = pack_bf16x2(__uint_as_float(r[8 * v + 0]) * inv, __uint_as_float(r[8 * v + 1]) * inv);
-              w.y = pack_bf16x2(__uint_as_float(r[8 * v + 2]) * inv, __uint_as_float(r[8 * v + 3]) * inv);
-              w.z = pack_bf16x2(__uint_as_float(r[8 * v + 4]) * inv, __uint_as_float(r[8 * v + 5]) * inv);
-              w.w = pack_bf16x2(__uint_as_float(r[8 * v + 6]) * inv, __uint_as_float(r[8 * v + 7]) * inv);
-              *reinterpret_cast<uint4*>(orow + 32 * c + 8 * v) = w;
+            for (int v = 0; v < 16; ++v)
+              w[v] = pack_bf16x2(__uint_as_float(r[2 * v]) * inv, __uint_as_float(r[2 * v + 1]) * inv);
+            bf16* o = e_out + 32 * c;
+            if (a.wide_out) {  // whole 32-byte sectors
+              st_global_v8(o, w);
+              st_global_v8(o + 16, w + 8);
+            } else {
+#pragma unroll
+              for (int v = 0; v < 4; ++v)
+                *reinterpret_cast<uint4*>(o + 8 * v) = make_uint4(w[4 * v], w[4 * v + 1], w[4 * v + 2], w[4 * v + 3]);
             }
           }
         }
-        if (q < a.N) a.lse2[(static_cast<size_t>(it.b) * a.Hq + h) * a.N + q] = m + log2f(l);
+        if (e_out != nullptr) *e_lse = e_m + log2f(e_l);
       }
       tc_fence_before();
-      arrive(&o_empty[x]);
+      arrive(&o_empty[x * NB + buf]);
+      ++n_e;
+    };
+    // The loop runs once more after the last item, for its epilogue.
+    PpItem it;
+    int r = 0;
+    while (true) {
+      int nk = 0;
+      while (nk == 0 && pp_next(r, a, it)) {
+        nk = x == 0 ? it.nk[0] : it.nk[1];
+        if (nk == 0) J += it.n_kb;
+      }
+      if (nk == 0 && n_e == n_o) break;
+      const int h = x == 0 ? it.h[0] : it.h[1];
+      const int w0 = (x == 0 ? it.qb[0] : it.qb[1]) * PP_BM + quad * 32;  // the warp's first query
+      const int q = w0 + lane;
+      const uint32_t o_addr = tmem + lane_off + o_col<HD>(x, n_o % NB);
+      float m = -INFINITY, l = 0.f;
+      int j = 0;
+      do {
+        if (nk > 0) {
+          ok = ok && __all_sync(0xffffffffu, mbar_wait_ab(&s_full[x], n_s & 1, a.status, abort_flag));
+          ++n_s;
+          tc_fence_after();
+          // keys k0 + e with e >= lim are hidden (causal diagonal, sequence end):
+          // lim grows with the row, so 32-column chunks below the first row's
+          // limit need no mask and chunks past the last row's hold no key
+          const int k0 = j * PP_BN;
+          const int keys = min(PP_BN, it.n - k0);
+          const int lim = a.causal ? min(keys, q - k0 + 1) : keys;
+          const int lim_first = a.causal ? min(keys, w0 - k0 + 1) : keys;
+          const int n_ch = ((a.causal ? min(keys, w0 + 32 - k0) : keys) + 31) / 32;
+          auto mask = [&](uint32_t (&v)[32], int c) {  // hidden scores become -inf
+            if (32 * c + 32 > lim_first) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] = 32 * c + e < lim ? v[e] : 0xff800000u;
+            }
+          };
+          if (keys & 15) {
+            // P is zero past the last key, but V's rows there belong to another
+            // sequence (or are zero-filled): keep a non-finite one out of 0 * V
+            const uint32_t va = smem_u32(sV + (J + j) % ST * TILE);
+            const int t = static_cast<int>(threadIdx.x) & 127, per = (-keys & 15) * 8;
+            for (int i = t; i < per * CH; i += 128)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(va + (i / per) * (PP_BN * 128) +
+                                                                          keys * 128 + (i % per) * 16),
+                           "r"(0)
+                           : "memory");
+            fence_proxy_async_smem();
+          }
+          if (ok && w0 < it.n) {  // some row of the warp is a query
+            // pass 1: the block's row maximum
+            float mx = -INFINITY;
+            int c1 = 0;
+#pragma unroll 1
+            for (; 32 * c1 + 64 <= lim_first; c1 += 2) {  // two whole chunks per TMEM round trip
+              uint32_t u[64];
+              tmem_ld32(s_addr + 32 * c1, *reinterpret_cast<uint32_t(*)[32]>(u));
+              tmem_ld32(s_addr + 32 * c1 + 32, *reinterpret_cast<uint32_t(*)[32]>(u + 32));
+              tmem_ld_wait();
+              float m4[4] = {mx, mx, mx, mx};
+#pragma unroll
+              for (int e = 0; e < 64; e += 8)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  m4[k] = fmax3(m4[k], __uint_as_float(u[e + 2 * k]), __uint_as_float(u[e + 2 * k + 1]));
+              mx = fmaxf(fmax3(m4[0], m4[1], m4[2]), m4[3]);
+            }
+#pragma unroll 1
+            for (int c = c1; c < n_ch; ++c) {
+              uint32_t u[32];
+              tmem_ld32(s_addr + 32 * c, u);
+              tmem_ld_wait();
+              mask(u, c);
+              float m4[4] = {mx, mx, mx, mx};
+#pragma unroll
+              for (int e = 0; e < 32; e += 8)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  m4[k] = fmax3(m4[k], __uint_as_float(u[e + 2 * k]), __uint_as_float(u[e + 2 * k + 1]));
+              mx = fmaxf(fmax3(m4[0], m4[1], m4[2]), m4[3]);
+            }
+            const float mb = mx == -INFINITY ? -INFINITY : mx * a.scale_log2;
+            const bool need = mb > m + PP_RESCALE_LOG2;
+            if (__any_sync(0xffffffffu, need)) {
+              const float mn = need ? mb : m;
+              const float f = need ? (m == -INFINITY ? 0.f : exp2f(m - mn)) : 1.f;
+              if (j > 0) {  // O holds blocks 0..j-1 (PV_x(j-1) finished before S_x(j) was signalled)
+#pragma unroll 1
+                for (int c = 0; c < HD / 32; ++c) {
+                  uint32_t v[32];
+                  tmem_ld32(o_addr + 32 * c, v);
+                  tmem_ld_wait();
+#pragma unroll
+                  for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * f);
+                  tmem_st32(o_addr + 32 * c, v);
+                }
+              }
+              l *= f;
+              m = mn;
+            }
+            // pass 2: P as a bf16 pair over the S columns just read; the next
+            // chunk's load is in flight while this one is converted
+            // P = 2^(s*scale - m) split as hi = P rounded to bf16 and lo = P - hi
+            // (exact in fp32, then rounded to bf16), so hi + lo carries P to
+            // about 17 bits
+            const uint64_t scale2 = f2pack(a.scale_log2, a.scale_log2);
+            const uint64_t nm2 = f2pack(-m, -m);
+            uint32_t v[32];
+            tmem_ld32(s_addr, v);
+            tmem_ld_wait();
+#pragma unroll 1
+            for (int c = 0; c < n_ch; ++c) {
+              mask(v, c);
+              uint64_t t[16];
+#pragma unroll
+              for (int e = 0; e < 16; ++e)
+                t[e] = ffma2(f2pack(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])), scale2, nm2);
+              if (c + 1 < n_ch) tmem_ld32(s_addr + 32 * (c + 1), v);
+              uint32_t hi[16], lo[16];
+              uint64_t lsum = f2pack(0.f, 0.f);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) {
+                float p0, p1, r0, r1;
+                f2unpack(t[e], p0, p1);
+                p0 = ex2_fast(p0);
+                p1 = ex2_fast(p1);
+                const uint64_t pp = f2pack(p0, p1);
+                lsum = fadd2(lsum, pp);
+                hi[e] = pack_bf16x2(p0, p1);
+                f2unpack(fsub2(pp, f2pack(bf16lo(hi[e]), bf16hi(hi[e]))), r0, r1);
+                lo[e] = pack_bf16x2(r0, r1);
+              }
+              float l0, l1;
+              f2unpack(lsum, l0, l1);
+              l += l0 + l1;
+              tmem_st16(s_addr + 32 * c, hi);
+              tmem_st16(s_addr + 32 * c + 16, lo);
+              tmem_ld_wait();
+            }
+            // P of the chunks that hold no key of this warp but some of the tile
+#pragma unroll 1
+            for (int c = n_ch; 32 * c < keys; ++c) {
+              const uint32_t z[16] = {};
+              tmem_st16(s_addr + 32 * c, z);
+              tmem_st16(s_addr + 32 * c + 16, z);
+            }
+            tmem_st_wait();
+          }
+          tc_fence_before();
+          arrive(&p_full[x]);
+        }
+        // the previous item's output, under this one's first P V
+        if (j == 0 && n_e < n_o) epilogue();
+      } while (++j < nk);
+      if (nk == 0) break;
+      const bool live = q < it.n;
+      e_out = live ? a.out + (static_cast<size_t>(it.row0) + q) * (static_cast<size_t>(a.Hq) * HD) + h * HD : nullptr;
+      e_lse = a.lse2 + (static_cast<size_t>(it.b) * a.Hq + h) * a.N + q;
+      e_m = m;
+      e_l = l;
+      ++n_o;
+      J += it.n_kb;
     }
   }
   tc_fence_before();
@@ -489,11 +653,12 @@ bool encode_rows(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows)
 
 template <int HD>
 cudaError_t run_pp(const void* qkv, int B, int N, int Hq, int Hkv, void* out, float* lse, int causal, int* status,
-                   cudaStream_t s) {
+                   cudaStream_t s, const int* cu, int rows) {
   using C = PpCfg<HD>;
   const int ld = (Hq + 2 * Hkv) * HD;
   CUtensorMap tm;
-  if (!encode_rows(&tm, qkv, static_cast<uint64_t>(ld), static_cast<uint64_t>(B) * N)) return cudaErrorInvalidValue;
+  if (!encode_rows(&tm, qkv, static_cast<uint64_t>(ld), cu ? static_cast<uint64_t>(rows) : static_cast<uint64_t>(B) * N))
+    return cudaErrorInvalidValue;
   static OncePerDevice once;
   const cudaError_t attr = set_smem_limit_once(once, attn_pp_kernel<HD>, static_cast<int>(C::SMEM));
   if (attr != cudaSuccess) return attr;
@@ -504,30 +669,37 @@ cudaError_t run_pp(const void* qkv, int B, int N, int Hq, int Hkv, void* out, fl
   a.N = N;
   a.Hq = Hq;
   a.Hkv = Hkv;
-  a.pairs = Hq / Hkv / 2;
   a.n_qb = (N + PP_BM - 1) / PP_BM;
   a.causal = causal;
+  // an even number of heads per group: two heads a tile pair (equal key blocks);
+  // otherwise two query blocks of one head
+  const int per = Hq / Hkv;
+  a.by_head = per % 2 == 0;
+  a.wide_out = (reinterpret_cast<uintptr_t>(out) & 31) == 0;
+  a.units = fast_div(a.by_head ? per / 2 : per);
+  a.groups = fast_div(Hkv);
+  a.inner = fast_div(B * Hkv * a.units.d);
+  a.total = (a.by_head ? a.n_qb : (a.n_qb + 1) / 2) * a.inner.d;
+  a.cu = cu;
   a.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(HD));
   a.status = status;
-  const int total = a.n_qb * B * Hkv * a.pairs;
-  const int grid = total < pp_sms() ? total : pp_sms();
+  const int grid = a.total < pp_sms() ? a.total : pp_sms();
   ZSAA_LAUNCH(attn_pp_kernel<HD>, dim3(grid), dim3(PP_THREADS), C::SMEM, s, tm, a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-bool attention_pp_supported(int dtype, int hd, int Hq, int Hkv, const int* cu, const uint8_t* key_alive,
-                            int* status) {
-  return dtype == ZSAA_BF16 && (hd == 64 || hd == 128) && Hkv > 0 && Hq % Hkv == 0 && (Hq / Hkv) % 2 == 0 &&
-         cu == nullptr && key_alive == nullptr && status != nullptr;
+bool attention_pp_supported(int dtype, int hd, int Hq, int Hkv, const uint8_t* key_alive, int* status) {
+  return dtype == ZSAA_BF16 && (hd == 64 || hd == 128) && Hkv > 0 && Hq % Hkv == 0 && key_alive == nullptr &&
+         status != nullptr;
 }
 
 cudaError_t launch_attention_pp(const void* qkv, int B, int N, int Hq, int Hkv, int hd, void* out, float* lse,
-                                int causal, int* status, cudaStream_t s) {
+                                int causal, int* status, cudaStream_t s, const int* cu, int rows) {
   if (B < 1 || N < 1) return cudaSuccess;
-  if (hd == 64) return run_pp<64>(qkv, B, N, Hq, Hkv, out, lse, causal, status, s);
-  if (hd == 128) return run_pp<128>(qkv, B, N, Hq, Hkv, out, lse, causal, status, s);
+  if (hd == 64) return run_pp<64>(qkv, B, N, Hq, Hkv, out, lse, causal, status, s, cu, rows);
+  if (hd == 128) return run_pp<128>(qkv, B, N, Hq, Hkv, out, lse, causal, status, s, cu, rows);
   return cudaErrorInvalidValue;
 }
 

@@ -66,25 +66,6 @@ struct CmCfg {
 };
 static_assert(CmCfg<64>::SMEM <= 227 * 1024 && CmCfg<128>::SMEM <= 227 * 1024, "shared memory");
 
-// n / d for 0 <= n < 2^31, d >= 1 (a tile's index is decoded by every role; a
-// plain division is a long dependent chain)
-struct FastDiv {
-  int d;
-  uint32_t m;  // about 2^32 / d
-  __device__ __forceinline__ int div(int n, int& rem) const {
-    int q = static_cast<int>(__umulhi(static_cast<uint32_t>(n), m));
-    rem = n - q * d;  // m is 2^32 / d rounded down: q is at most one short
-    if (rem >= d) {
-      ++q;
-      rem -= d;
-    }
-    return q;
-  }
-};
-FastDiv fast_div(int d) {
-  return FastDiv{d, d == 1 ? 0xffffffffu : static_cast<uint32_t>((1ull << 32) / static_cast<uint32_t>(d))};
-}
-
 struct CmArgs {
   const float* lse2;   // [B, Hq, N]
   const float* vnorm;  // [B*N, Hkv] ||v|| per row and group (used when weight_vnorm)

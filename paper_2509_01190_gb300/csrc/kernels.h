@@ -146,33 +146,20 @@ cudaError_t launch_gemm_f32(const float* A, int lda, const TcWeights& W, int epi
                             cudaStream_t s);
 
 // ---- attention (k_attn.cu)
-// Two-tile tcgen05 attention (k_attn_pp.cu) for bf16 heads of 64 or 128 dims,
-// fixed lengths, an even number of query heads per KV head: persistent CTAs
-// walk (sequence, KV group, pair of query heads, 128 queries) items, O kept
-// in TMEM, V read from the qkv rows.  Same outputs as launch_attention;
-// bounded waits report through status.
-bool attention_pp_supported(int dtype, int hd, int Hq, int Hkv, const int* cu, const uint8_t* key_alive,
-                            int* status);
+// Two-tile tcgen05 attention (k_attn_pp.cu) for bf16 heads of 64 or 128 dims:
+// persistent CTAs walk items of two 128-query tiles that share keys (two heads
+// of a group, or two query blocks of a head), O kept in TMEM, V read from the
+// qkv rows.  Same outputs as launch_attention; bounded waits report through
+// status.  cu: packed sequences of different lengths, rows [cu[b], cu[b+1])
+// of `rows` in all; N is then the longest length (and the stride of lse).
+bool attention_pp_supported(int dtype, int hd, int Hq, int Hkv, const uint8_t* key_alive, int* status);
 cudaError_t launch_attention_pp(const void* qkv, int B, int N, int Hq, int Hkv, int hd, void* out, float* lse,
-                                int causal, int* status, cudaStream_t s);
-// tcgen05 attention (k_attn_tc.cu) for bf16 heads of 64 or 128 dims, fixed
-// lengths: a transpose kernel writes V^T into vt (attention_tc_vt_elems bf16
-// elements), then persistent CTAs walk (128 queries, head, sequence) items.
-// Same outputs as launch_attention; bounded waits report through status.
-bool attention_tc_supported(int dtype, int hd, const int* cu, const uint8_t* key_alive, int* status,
-                            void* vt);
-size_t attention_tc_vt_elems(int B, int N, int Hkv, int hd);
-constexpr int kAttentionTcMinN = 256;
-bool attention_tc_preferred(int N);
-cudaError_t launch_attention_tc(const void* qkv, void* vt, int B, int N, int Hq, int Hkv, int hd, void* out,
-                                float* lse, int causal, int* status, cudaStream_t s);
+                                int causal, int* status, cudaStream_t s, const int* cu = nullptr, int rows = 0);
 // causal = 0: bidirectional (Eq. 1 with M = 0); the column-mass kernels below
 // take the same flag.
-// cu (bf16 only): packed sequences of different lengths, rows [cu[b], cu[b+1]);
-// N is then the longest length (grid size and the stride of lse).
 cudaError_t launch_attention(int dtype, const void* qkv, int B, int N, int Hq, int Hkv, int hd,
                              void* out, float* lse, int causal, cudaStream_t s,
-                             const int* cu = nullptr, const uint8_t* key_alive = nullptr);
+                             const uint8_t* key_alive = nullptr);
 // key_alive (bf16, fixed length): [B, N] flags of the masked mode; keys with 0
 // are hidden from every query.
 // fp32 tiled kernels (k_attn_f32.cu): heads of 32, 64 or 128 dims, 16-byte

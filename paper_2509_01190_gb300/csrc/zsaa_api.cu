@@ -314,7 +314,6 @@ struct zsaa_model {
   void* attn = nullptr;
   void* act = nullptr;
   float* lse = nullptr;
-  void* vt = nullptr;        // V^T of the current layer for the tcgen05 attention (bf16, hd 64)
   float* colmass = nullptr;  // query-chunk partials of the column mass / scores
   float* vnorm = nullptr;    // ||v|| per row and KV group, from the QKV epilogue (bf16)
   float* scores = nullptr;
@@ -471,7 +470,7 @@ void free_model(zsaa_model* m) {
   if (m->side) cudaStreamDestroy(m->side);
   if (m->ev_fork) cudaEventDestroy(m->ev_fork);
   if (m->ev_join) cudaEventDestroy(m->ev_join);
-  void* ptrs[] = {m->h[0], m->h[1], m->x, m->qkv, m->attn, m->act, m->lse, m->vt, m->colmass, m->vnorm,
+  void* ptrs[] = {m->h[0], m->h[1], m->x, m->qkv, m->attn, m->act, m->lse, m->colmass, m->vnorm,
                   m->scores, m->idx, m->pos[0], m->pos[1], m->rope_cos, m->rope_sin,
                   m->splitk_ws, m->splitk_flags, m->status, m->stage_tok, m->stage_logits,
                   m->stage_pos};
@@ -627,11 +626,8 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
     {
       const double pairs = static_cast<double>(B) * Hq * n_pairs(N);
       TRACE("attention", 4.0 * pairs * hd, Md * (m->ld_qkv + m->dq) * es + static_cast<double>(B) * Hq * N * 4.0);
-      if (attention_pp_supported(dt, hd, Hq, Hkv, nullptr, nullptr, m->status)) {
+      if (attention_pp_supported(dt, hd, Hq, Hkv, nullptr, m->status)) {
         ZCK(launch_attention_pp(m->qkv, B, N, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s));
-      } else if (attention_tc_supported(dt, hd, nullptr, nullptr, m->status, m->vt) && attention_tc_preferred(N)) {
-        trace_scope_.kernels = 2;  // V transpose + attention
-        ZCK(launch_attention_tc(m->qkv, m->vt, B, N, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s));
       } else {
         ZCK(launch_attention(dt, m->qkv, B, N, Hq, Hkv, hd, m->attn, m->lse, causal, s));
       }
@@ -917,8 +913,12 @@ zsaa_status run_forward_masked(zsaa_model* m, const int32_t* tok, int B, int L, 
     }
     {
       TRACE("attention", 4.0 * pairs * hd, Md * (m->ld_qkv + m->dq) * es + static_cast<double>(B) * Hq * L * 4.0);
-      ZCK(launch_attention(dt, m->qkv, B, L, Hq, Hkv, hd, m->attn, m->lse, causal, s, nullptr,
-                           reactivate ? nullptr : m->alive));
+      if (reactivate && attention_pp_supported(dt, hd, Hq, Hkv, nullptr, m->status)) {  // nothing is hidden
+        ZCK(launch_attention_pp(m->qkv, B, L, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s));
+      } else {
+        ZCK(launch_attention(dt, m->qkv, B, L, Hq, Hkv, hd, m->attn, m->lse, causal, s,
+                             reactivate ? nullptr : m->alive));
+      }
     }
     // O-projection beside the column mass and selection (see run_forward);
     // the MLP's RMSNorm joins it
@@ -1151,7 +1151,7 @@ zsaa_status run_forward_varlen(zsaa_model* m, const int32_t* tok, const int32_t*
         pairs += causal ? nb * (nb + 1) / 2.0 : nb * nb;
       }
       TRACE("attention", 4.0 * pairs * Hq * hd, Md * (m->ld_qkv + m->dq) * es + static_cast<double>(B) * Hq * Nm * 4.0);
-      ZCK(launch_attention(dt, m->qkv, B, Nm, Hq, Hkv, hd, m->attn, m->lse, causal, s, cu_dev(li)));
+      ZCK(launch_attention_pp(m->qkv, B, Nm, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s, cu_dev(li), M));
     }
     // O-projection beside the column mass and selection (see run_forward)
     const bool fork = !m->tracing && prunes(c, l) && rows[l] < M && Nm <= kSelectPartsMaxN;
@@ -1657,8 +1657,6 @@ zsaa_status zsaa_model_create(const zsaa_config* cfg, const zsaa_weights* w, int
   alloc(&m->attn, rows * m->dq * esz);
   alloc(&m->act, rows * F * esz);
   alloc(reinterpret_cast<void**>(&m->lse), rows * cfg->n_heads * sizeof(float));
-  if (cfg->dtype == ZSAA_BF16 && (cfg->head_dim == 64 || cfg->head_dim == 128))
-    alloc(&m->vt, attention_tc_vt_elems(max_B, max_L, cfg->n_kv_heads, cfg->head_dim) * 2);
   alloc(reinterpret_cast<void**>(&m->colmass),
         colmass_parts_elems(max_B, max_L, cfg->n_heads, cfg->n_kv_heads) * sizeof(float));
   alloc(reinterpret_cast<void**>(&m->vnorm), rows * cfg->n_kv_heads * sizeof(float));
@@ -1879,17 +1877,8 @@ zsaa_status zsaa_op_attention_ex(const void* qkv, int B, int N, int Hq, int Hkv,
   if (dtype == ZSAA_F32 && (hd < 1 || hd > 128)) return fail(ZSAA_ERR_UNSUPPORTED, "f32 attention needs hd <= 128");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int* status = shared_status();
-  if (attention_pp_supported(dtype, hd, Hq, Hkv, nullptr, nullptr, status)) {
+  if (attention_pp_supported(dtype, hd, Hq, Hkv, nullptr, status)) {
     ZCK(launch_attention_pp(qkv, B, N, Hq, Hkv, hd, out, lse, causal ? 1 : 0, status, s));
-    return ZSAA_OK;
-  }
-  if (dtype == ZSAA_BF16 && status != nullptr) {  // the one-tile tcgen05 kernel, V^T scratch
-    void* vt = nullptr;
-    ZCK(cudaMallocAsync(&vt, attention_tc_vt_elems(B, N, Hkv, hd) * 2, s));
-    cudaError_t e = launch_attention_tc(qkv, vt, B, N, Hq, Hkv, hd, out, lse, causal ? 1 : 0, status, s);
-    cudaError_t e2 = cudaFreeAsync(vt, s);
-    ZCK(e);
-    ZCK(e2);
     return ZSAA_OK;
   }
   ZCK(launch_attention(dtype, qkv, B, N, Hq, Hkv, hd, out, lse, causal ? 1 : 0, s));
