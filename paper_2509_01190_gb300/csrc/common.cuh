@@ -65,6 +65,18 @@ __device__ __forceinline__ void pdl_trigger() {
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A pointer to data that an earlier kernel on the stream writes, to be used only
+// after pdl_wait: the compiler may move a load through a `const __restrict__`
+// parameter above the wait (it takes such memory as never written while the
+// kernel runs), where a kernel that was launched early reads the old values.  A
+// load through the value returned here depends on this statement, which stays
+// after the wait.
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p) : : "memory");
+  return p;
+}
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        Args&&... args) {

@@ -55,6 +55,8 @@ __global__ void __launch_bounds__(128)
                          int causal, const uint8_t* __restrict__ key_alive) {
   pdl_trigger();
   pdl_wait();
+  qkv = after_wait(qkv);
+  key_alive = after_wait(key_alive);
   constexpr int ROWB = HD * 2;
   constexpr int TILE = 64 * ROWB;
   extern __shared__ __align__(128) uint8_t sm[];
@@ -231,6 +233,8 @@ __global__ void __launch_bounds__(128)
                         float* __restrict__ parts, float scale_log2, int causal) {
   pdl_trigger();
   pdl_wait();
+  qkv = after_wait(qkv);
+  lse2 = after_wait(lse2);
   constexpr int ROWB = HD * 2;
   constexpr int TILE = 64 * ROWB;
   extern __shared__ __align__(128) uint8_t sm[];
@@ -365,6 +369,7 @@ __global__ void colmass_reduce_kernel(const float* __restrict__ parts, int n_qc,
                                       int N, int sum_groups, float* __restrict__ out) {
   pdl_trigger();
   pdl_wait();
+  parts = after_wait(parts);
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int total = sum_groups ? B * N : B * G * N;
   if (idx >= total) return;
@@ -386,6 +391,7 @@ __global__ void attn_fwd_f32_kernel(const float* __restrict__ qkv, int N, int Hq
                                     float scale_log2, int causal) {
   pdl_trigger();
   pdl_wait();
+  qkv = after_wait(qkv);
   const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int h = blockIdx.y, b = blockIdx.z, lane = threadIdx.x & 31;
   if (i >= N) return;
@@ -442,6 +448,8 @@ __global__ void colmass_f32_kernel(const float* __restrict__ qkv, const float* _
                                    float* __restrict__ parts, float scale_log2, int causal) {
   pdl_trigger();
   pdl_wait();
+  qkv = after_wait(qkv);
+  lse2 = after_wait(lse2);
   const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int g = blockIdx.y, b = blockIdx.z, lane = threadIdx.x & 31;
   if (j >= N) return;

@@ -89,6 +89,8 @@ __global__ void __launch_bounds__(AF_THREADS)
     attn_f32_tile_kernel(const float* __restrict__ qkv, int N, int Hq, int Hkv, float* __restrict__ out,
                          float* __restrict__ lse2, float scale_log2, int causal) {
   pdl_trigger();
+  pdl_wait();
+  qkv = after_wait(qkv);
   constexpr int BQ = 8 * R, LD = af_ld<HD>();
   constexpr int NP = HD / 32;  // pairs of output dims a thread owns per row
   extern __shared__ __align__(16) float sm[];
@@ -106,7 +108,6 @@ __global__ void __launch_bounds__(AF_THREADS)
   const int q0 = qb * BQ;
   const int n_keys = causal ? min(N, q0 + BQ) : N;
   const int n_kb = (n_keys + AF_COLS - 1) / AF_COLS;
-  pdl_wait();
   af_load<HD>(sQ, base + h * HD, ld, q0, BQ, N);
   af_load<HD>(sK, Kg, ld, 0, AF_COLS, N);
   cp_async_commit();
@@ -225,6 +226,9 @@ __global__ void __launch_bounds__(AF_THREADS)
                             int Hkv, int B, int weight_vnorm, float* __restrict__ parts, float scale_log2,
                             int causal) {
   pdl_trigger();
+  pdl_wait();
+  qkv = after_wait(qkv);
+  lse2 = after_wait(lse2);
   constexpr int BK = 8 * R, LD = af_ld<HD>();
   extern __shared__ __align__(16) float sm[];
   float* sK = sm;
@@ -238,7 +242,6 @@ __global__ void __launch_bounds__(AF_THREADS)
   const float* L = lse2 + (static_cast<size_t>(b) * Hq + h) * N;
   const int j0 = kb * BK;
   const int qb0 = causal ? j0 / AF_COLS : 0, n_qb = (N + AF_COLS - 1) / AF_COLS;
-  pdl_wait();
   auto issue = [&](int qb, int buf) {
     af_load<HD>(sQ + buf * AF_COLS * LD, base + h * HD, ld, qb * AF_COLS, AF_COLS, N);
     if (tid < AF_COLS) {

@@ -26,6 +26,8 @@ __global__ void kv_write_kernel(const bf16* __restrict__ qkv, int ld,
                                 int hd, KvLayer c) {
   pdl_trigger();
   pdl_wait();
+  qkv = after_wait(qkv);
+  pos = after_wait(pos);
   const int cpr = hd / 8;
   const long long total = static_cast<long long>(B) * N * 2 * Hkv * cpr;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
@@ -76,6 +78,8 @@ __global__ void __launch_bounds__(decode_warps<HD, PER>() * 32)
   const int g = blockIdx.x, b = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_wait();
+  qkv32 = after_wait(qkv32);
+  step = after_wait(step);
   const int t = *step;
   const int p = L0 + t;
   const int row = c.base + t;

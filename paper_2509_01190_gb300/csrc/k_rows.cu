@@ -25,6 +25,7 @@ __global__ void embed_kernel(const uint4* __restrict__ E, const int32_t* __restr
                              int32_t* __restrict__ pos, int* status) {
   pdl_trigger();
   pdl_wait();
+  tok = after_wait(tok);
   const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -55,6 +56,7 @@ __global__ void rmsnorm_kernel(const T* __restrict__ h, const T* __restrict__ w,
                                float eps, T* __restrict__ x) {
   pdl_trigger();
   pdl_wait();
+  h = after_wait(h);
   const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -87,6 +89,7 @@ __global__ void rmsnorm_bf16_reg_kernel(const uint4* __restrict__ h, const uint4
   pdl_trigger();
   stage_norm_weights(w, vec, sw);
   pdl_wait();
+  h = after_wait(h);
   const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -138,6 +141,7 @@ __global__ void rmsnorm_bf16_vec_kernel(const uint4* __restrict__ h, const uint4
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 32) prefetch_norm_weights(w, vec_per_row, lane);
   pdl_wait();
+  h = after_wait(h);
   if (r >= rows) return;
   const uint4* hr = h + static_cast<size_t>(r) * vec_per_row;
   uint4* xr = x + static_cast<size_t>(r) * vec_per_row;
@@ -173,6 +177,7 @@ __global__ void row_norm_bf16_kernel(const uint4* __restrict__ h, int rows, int 
                                      float* __restrict__ s) {
   pdl_trigger();
   pdl_wait();
+  h = after_wait(h);
   const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -212,6 +217,7 @@ __global__ void row_norm_f32_kernel(const float* __restrict__ h, int rows, int d
                                     float* __restrict__ s) {
   pdl_trigger();
   pdl_wait();
+  h = after_wait(h);
   const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -254,6 +260,8 @@ __global__ void __launch_bounds__(THREADS)
                        const int* __restrict__ cu_out, uint8_t* __restrict__ alive) {
   pdl_trigger();
   pdl_wait();
+  scores = after_wait(scores);
+  parts = after_wait(parts);
   const int b = blockIdx.x;
   // fixed length: N = Ns rows in, k = ks kept per sequence; variable length
   // (FROM_PARTS only): this sequence's counts from the packed row offsets,
@@ -447,6 +455,7 @@ __global__ void flags_from_idx_kernel(const int32_t* __restrict__ idx, int N, in
                                       uint8_t* __restrict__ flags, int* status) {
   pdl_trigger();
   pdl_wait();
+  idx = after_wait(idx);
   uint8_t* f = flags + static_cast<size_t>(blockIdx.x) * N;
   for (int j = threadIdx.x; j < N; j += blockDim.x) f[j] = 0;
   __syncthreads();
@@ -470,6 +479,9 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ src, int N, int k, 
                                    int total, int* status) {
   pdl_trigger();
   pdl_wait();
+  src = after_wait(src);
+  idx = after_wait(idx);
+  pos_in = after_wait(pos_in);
   const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= total) return;
@@ -517,6 +529,10 @@ __global__ void rows_norm_bf16_kernel(const uint4* __restrict__ src, const int32
   const int lane = threadIdx.x & 31;
   stage_norm_weights(w, vec, sw);
   pdl_wait();
+  src = after_wait(src);
+  tok = after_wait(tok);
+  idx = after_wait(idx);
+  pos_in = after_wait(pos_in);
   if (r >= rows) return;
   size_t srow;
   int p;
@@ -594,6 +610,7 @@ __global__ void rope_f32_kernel(float* __restrict__ qkv, int rows, int ld, int r
                                 const float* __restrict__ sin_t) {
   pdl_trigger();
   pdl_wait();
+  pos = after_wait(pos);
   const int r = blockIdx.y;
   const int half = hd / 2;
   const int pairs = rope_cols / 2;
@@ -618,6 +635,7 @@ __global__ void cls_head_kernel(const T* __restrict__ h, int N, int d,
                                 int n_classes, float* __restrict__ out, const int* __restrict__ cu) {
   pdl_trigger();
   pdl_wait();
+  h = after_wait(h);
   extern __shared__ float xs[];  // d floats
   __shared__ float red[32];
   const int b = blockIdx.x;

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 16 ? 1 : 2)
       }
       if (!waited) {  // activations come from the previous kernel
         pdl_wait();
+        A = after_wait(A);
         waited = true;
       }
 #pragma unroll
