@@ -53,6 +53,24 @@ __global__ void kv_write_kernel(const bf16* __restrict__ qkv, int ld,
   }
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+template <int N>
+__device__ __forceinline__ void load_floats(const float* p, float (&v)[N]) {
+  if constexpr (N % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 u = *reinterpret_cast<const float4*>(p + i);
+      v[i] = u.x, v[i + 1] = u.y, v[i + 2] = u.z, v[i + 3] = u.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = p[i];
+  }
+}
+
 // One CTA per (KV group, sequence): RoPE and bf16 rounding of the group's PER
 // query heads and of its key, append of key/value to the cache, then Eq. 1 of
 // the PER queries over the cached rows.  8 warps take interleaved blocks of 32
@@ -75,17 +93,58 @@ __global__ void __launch_bounds__(decode_warps<HD, PER>() * 32)
   constexpr int W = decode_warps<HD, PER>();
   __shared__ float wm[W][PER], wl[W][PER];
   __shared__ float wacc[W][PER][HD];
+  __shared__ __align__(16) float ps[W][32][PER];
   const int g = blockIdx.x, b = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // Between two uses of a layer's cache and of the RoPE row a step's weights
+  // pass through L2, so both come from HBM: ask for them before the wait.  (A
+  // hint only: a step counter that is about to move names the previous row.)
+  {
+    const size_t at = (static_cast<size_t>(b) * Hkv + g) * c.cap * static_cast<size_t>(HD);
+    const int lines = c.base * HD / 64;  // 128-byte lines of the prefill's rows
+    for (int i = threadIdx.x; i < 2 * lines; i += blockDim.x) {
+      const bf16* base = static_cast<const bf16*>(i < lines ? c.k : c.v) + at;
+      prefetch_l2(base + static_cast<size_t>(i < lines ? i : i - lines) * 64);
+    }
+    const size_t p_row = static_cast<size_t>(L0 + *reinterpret_cast<const volatile int*>(step)) * HALF;
+    if (threadIdx.x < 2 * HALF / 32) {
+      const int i = threadIdx.x;
+      prefetch_l2((i < HALF / 32 ? cos_t : sin_t) + p_row + (i % (HALF / 32)) * 32);
+    }
+  }
   pdl_wait();
   qkv32 = after_wait(qkv32);
   step = after_wait(step);
+  // A lane's key row of a 32-key block and its head-dim slice of the block's 32
+  // value rows (rows past nb - 1 repeat row 0), all requested together.
+  uint4 kr[HD / 8];
+  uint32_t vw[32][DPL / 2];
+  auto load_block = [&](const bf16* Kc, const bf16* Vc, int j0, int nb) {
+    const uint4* k4 = reinterpret_cast<const uint4*>(Kc + static_cast<size_t>(j0 + (lane < nb ? lane : 0)) * HD);
+#pragma unroll
+    for (int ch = 0; ch < HD / 8; ++ch) kr[ch] = k4[ch];
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) {
+      const bf16* vr = Vc + static_cast<size_t>(j0 + (jj < nb ? jj : 0)) * HD + lane * DPL;
+      if constexpr (DPL == 2) {
+        vw[jj][0] = *reinterpret_cast<const uint32_t*>(vr);
+      } else {
+        const uint2 w = *reinterpret_cast<const uint2*>(vr);
+        vw[jj][0] = w.x;
+        vw[jj][1] = w.y;
+      }
+    }
+  };
+  bf16* Kc = static_cast<bf16*>(c.k) + (static_cast<size_t>(b) * Hkv + g) * c.cap * static_cast<size_t>(HD);
+  bf16* Vc = static_cast<bf16*>(c.v) + (static_cast<size_t>(b) * Hkv + g) * c.cap * static_cast<size_t>(HD);
+  // the warp's first block, when it is all prefill rows: its round trip runs
+  // under the step counter's, the projections' and the rotation
+  bool loaded = warp * 32 + 32 <= c.base;
+  if (loaded) load_block(Kc, Vc, warp * 32, 32);
   const int t = *step;
   const int p = L0 + t;
   const int row = c.base + t;
   const float* src = qkv32 + static_cast<size_t>(b) * ld;
-  bf16* Kc = static_cast<bf16*>(c.k) + (static_cast<size_t>(b) * Hkv + g) * c.cap * static_cast<size_t>(HD);
-  bf16* Vc = static_cast<bf16*>(c.v) + (static_cast<size_t>(b) * Hkv + g) * c.cap * static_cast<size_t>(HD);
 
   for (int i = threadIdx.x; i < (PER + 1) * HALF; i += blockDim.x) {
     const int h = i / HALF, dd = i % HALF;  // h < PER: query head g*PER + h; h == PER: key head g
@@ -121,26 +180,13 @@ __global__ void __launch_bounds__(decode_warps<HD, PER>() * 32)
   for (int j0 = warp * 32; j0 < n_keys; j0 += W * 32) {
     const int j = j0 + lane;
     const int nb = min(32, n_keys - j0);
-    // this lane's head-dim slice of the block's 32 value rows, requested with
-    // the key row below so that both memory latencies overlap
-    uint32_t vw[32][DPL / 2];
-#pragma unroll
-    for (int jj = 0; jj < 32; ++jj) {
-      const bf16* vr = Vc + static_cast<size_t>(j0 + (jj < nb ? jj : 0)) * HD + lane * DPL;
-      if constexpr (DPL == 2) {
-        vw[jj][0] = *reinterpret_cast<const uint32_t*>(vr);
-      } else {
-        const uint2 w = *reinterpret_cast<const uint2*>(vr);
-        vw[jj][0] = w.x;
-        vw[jj][1] = w.y;
-      }
-    }
+    if (!loaded) load_block(Kc, Vc, j0, nb);
+    loaded = false;
     float sc[PER];
     if (j < n_keys) {
       float dot[PER];
 #pragma unroll
       for (int h = 0; h < PER; ++h) dot[h] = 0.f;
-      const uint4* kr = reinterpret_cast<const uint4*>(Kc + static_cast<size_t>(j) * HD);
 #pragma unroll
       for (int ch = 0; ch < HD / 8; ++ch) {
         const uint4 kv = kr[ch];
@@ -176,23 +222,28 @@ __global__ void __launch_bounds__(decode_warps<HD, PER>() * 32)
       for (int e = 0; e < DPL; ++e) acc[h][e] *= corr;
       m[h] = mn;
     }
+    // P V: the block's probabilities through shared memory, PER of a key at a
+    // time to every lane (a shuffle per key and head took several times as long)
+#pragma unroll
+    for (int h = 0; h < PER; ++h) ps[warp][lane][h] = pj[h];
+    __syncwarp();
 #pragma unroll
     for (int jj = 0; jj < 32; ++jj) {
       if (jj < nb) {  // warp-uniform
-        float vv[DPL];
+        float vv[DPL], pk[PER];
+        load_floats<PER>(ps[warp][jj], pk);
 #pragma unroll
         for (int e2 = 0; e2 < DPL / 2; ++e2) {
           vv[2 * e2] = __uint_as_float(vw[jj][e2] << 16);
           vv[2 * e2 + 1] = __uint_as_float(vw[jj][e2] & 0xffff0000u);
         }
 #pragma unroll
-        for (int h = 0; h < PER; ++h) {
-          const float pk = __shfl_sync(0xffffffffu, pj[h], jj);
+        for (int h = 0; h < PER; ++h)
 #pragma unroll
-          for (int e = 0; e < DPL; ++e) acc[h][e] = fmaf(pk, vv[e], acc[h][e]);
-        }
+          for (int e = 0; e < DPL; ++e) acc[h][e] = fmaf(pk[h], vv[e], acc[h][e]);
       }
     }
+    __syncwarp();  // ps is rewritten by the next block
   }
   if (lane == 0) {
 #pragma unroll

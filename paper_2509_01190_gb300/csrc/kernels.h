@@ -76,6 +76,15 @@ struct GemmParams {
   int* splitk_flags;    // kMaxGemmCtas * 4 ints, zero before the first launch
   int w_const;          // fp32: no kernel writes W, so it may be read before the previous kernel ends
   int* launches;        // optional host counter: kernels launched are added to it
+  // Weight-streaming kernel only: with norm_w, A holds residual rows that are
+  // RMS-normed first (their sums of squares per 16 columns in norm_ss
+  // [K/16][16]); with norm_ss_out (kEpiResid) those of the rows written;
+  // advance: a counter to step, after the previous kernels have ended (with norm_w).
+  const void* norm_w;
+  const float* norm_ss;
+  float norm_eps;
+  float* norm_ss_out;   // [N/16][16]
+  int* advance;
   float* vnorm_out;     // kEpiRope: if set, ||v|| of each row's value heads, [M, (N - rope_cols) / hd]
 };
 
@@ -119,6 +128,8 @@ int gemm_tc_schedule(int epi, int M, int N, int K, int hd, int sms, int pair_slo
 // A and W.  launch_gemm_tc routes such calls here.
 constexpr int kSkinnyMaxM = 16;
 bool skinny_supported(const void* A, int lda, const TcWeights& W, int epi, const GemmParams& p);
+// Whether M rows of K columns can be normed in it (GemmParams::norm_w).
+bool skinny_norm_supported(int M, int K);
 cudaError_t launch_gemm_skinny(const void* A, int lda, const TcWeights& W, int epi,
                                const GemmParams& p, cudaStream_t s);
 

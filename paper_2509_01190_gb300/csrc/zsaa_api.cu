@@ -378,6 +378,7 @@ struct zsaa_cache {
   size_t kv_bytes = 0, kv_bytes_unpruned = 0;
   float* rope_cos = nullptr;             // [L + max_new, hd/2]
   float* rope_sin = nullptr;
+  float* norm_ss = nullptr;              // [2][d/16][16] sums of squares of the residual rows (see run_decode)
   float* qkv32 = nullptr;                // [B, ld_qkv] float32 projections of the new rows
   int32_t* last_idx = nullptr;           // [B]: N_n - 1, the last kept row
   int* step = nullptr;                   // device: tokens generated since the prefill
@@ -1432,7 +1433,7 @@ void rope_host_table(double theta, int hd, int n_pos, std::vector<float>* cs, st
 void free_cache(zsaa_cache* c) {
   if (c == nullptr) return;
   if (c->graph) cudaGraphExecDestroy(c->graph);
-  void* ptrs[] = {c->kv, c->pos, c->rope_cos, c->rope_sin, c->qkv32, c->last_idx, c->step};
+  void* ptrs[] = {c->kv, c->pos, c->rope_cos, c->rope_sin, c->qkv32, c->norm_ss, c->last_idx, c->step};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete c;
@@ -1447,6 +1448,17 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
   const double es = static_cast<double>(m->esz), Bd = B;
   void* h = m->h[0];
   zsaa_status st = ZSAA_OK;
+  // Few enough rows for the weight-streaming kernel: the residual projections
+  // leave the rows' sums of squares and the next projection norms the rows
+  // itself, so only the embedding's norm is a kernel of its own; the head's
+  // kernel steps the position.
+  const bool fuse = skinny_norm_supported(B, d) && reinterpret_cast<uintptr_t>(m->head) % 16 == 0;
+  float* ss[2] = {kc->norm_ss, kc->norm_ss + d};  // after the attention branch, after the MLP branch
+  auto normed = [&](GemmParams& p, const void* w, const float* sums) {
+    p.norm_w = w;
+    p.norm_ss = sums;
+    p.norm_eps = c.rms_eps;
+  };
 #define TRACE(name, fl, by) TraceScope trace_scope_(m, name, fl, by, s)
   {
     TRACE("embed_norm", 0.0, Bd * (3.0 * d * es + 8.0));
@@ -1454,7 +1466,8 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
                          LW(m, 0, kAttnNorm), c.rms_eps, h, m->x, m->pos[0], m->status, s));
   }
   for (int li = 0; li < c.n_layers; ++li) {
-    if (li > 0) {
+    const bool in_norm = fuse && li > 0;  // layer 0's rows come normed from the embedding
+    if (li > 0 && !fuse) {
       TRACE("rmsnorm", 0.0, 2.0 * Bd * d * es);
       ZCK(launch_rmsnorm(c.dtype, h, LW(m, li, kAttnNorm), B, d, c.rms_eps, m->x, s));
     }
@@ -1465,10 +1478,11 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
       p.K = d;
       p.out = kc->qkv32;
       p.ldo = m->ld_qkv;
+      if (in_norm) normed(p, LW(m, li, kAttnNorm), ss[1]);
       TcWeights W{LW(m, li, kWq), LW(m, li, kWk), LW(m, li, kWv), m->dq, m->dq + m->dkv};
       TRACE("gemm_qkv", 2.0 * Bd * m->ld_qkv * d, (Bd * d + static_cast<double>(m->ld_qkv) * d) * es + Bd * m->ld_qkv * 4.0);
       trace_scope_.kernels = 0;
-      st = linear(m, m->x, d, W, kEpiStoreF32, p, s, &trace_scope_.kernels);
+      st = linear(m, in_norm ? h : m->x, d, W, kEpiStoreF32, p, s, &trace_scope_.kernels);
       if (st != ZSAA_OK) return st;
     }
     {
@@ -1486,13 +1500,14 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
       q.out = h;
       q.ldo = d;
       q.resid = h;
+      if (fuse) q.norm_ss_out = ss[0];
       TcWeights W{LW(m, li, kWo), nullptr, nullptr, d, d};
       TRACE("gemm_o_resid", 2.0 * Bd * d * m->dq, (Bd * m->dq + static_cast<double>(d) * m->dq + 2.0 * Bd * d) * es);
       trace_scope_.kernels = 0;
       st = linear(m, m->attn, m->dq, W, kEpiResid, q, s, &trace_scope_.kernels);
       if (st != ZSAA_OK) return st;
     }
-    {
+    if (!fuse) {
       TRACE("rmsnorm", 0.0, 2.0 * Bd * d * es);
       ZCK(launch_rmsnorm(c.dtype, h, LW(m, li, kMlpNorm), B, d, c.rms_eps, m->x, s));
     }
@@ -1504,10 +1519,11 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
       q.K = d;
       q.out = m->act;
       q.ldo = c.ffn_dim;
+      if (fuse) normed(q, LW(m, li, kMlpNorm), ss[0]);
       TcWeights W{LW(m, li, kWg), LW(m, li, kWu), nullptr, c.ffn_dim, c.ffn_dim};
       TRACE("gemm_gate_up_swiglu", 4.0 * Bd * F * d, (Bd * d + 2.0 * F * d + Bd * F) * es);
       trace_scope_.kernels = 0;
-      st = linear(m, m->x, d, W, kEpiSwiGLU, q, s, &trace_scope_.kernels);
+      st = linear(m, fuse ? h : m->x, d, W, kEpiSwiGLU, q, s, &trace_scope_.kernels);
       if (st != ZSAA_OK) return st;
     }
     {
@@ -1518,6 +1534,7 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
       q.out = h;
       q.ldo = d;
       q.resid = h;
+      if (fuse) q.norm_ss_out = ss[1];
       TcWeights W{LW(m, li, kWd), nullptr, nullptr, d, d};
       TRACE("gemm_down_resid", 2.0 * Bd * d * F, (Bd * F + F * d + 2.0 * Bd * d) * es);
       trace_scope_.kernels = 0;
@@ -1525,7 +1542,7 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
       if (st != ZSAA_OK) return st;
     }
   }
-  {
+  if (!fuse) {
     TRACE("rmsnorm", 0.0, 2.0 * Bd * d * es);
     ZCK(launch_rmsnorm(c.dtype, h, m->final_norm, B, d, c.rms_eps, m->x, s));
   }
@@ -1536,14 +1553,18 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
     q.K = d;
     q.out = logits;
     q.ldo = c.vocab;
+    if (fuse) {
+      normed(q, m->final_norm, ss[1]);
+      q.advance = kc->step;
+    }
     TcWeights W{m->head, nullptr, nullptr, c.vocab, c.vocab};
     const double V = c.vocab;
     TRACE("gemm_lm_head", 2.0 * Bd * V * d, (Bd * d + V * d) * es + Bd * V * 4.0);
     trace_scope_.kernels = 0;
-    st = linear(m, m->x, d, W, kEpiStoreF32, q, s, &trace_scope_.kernels);
+    st = linear(m, fuse ? h : m->x, d, W, kEpiStoreF32, q, s, &trace_scope_.kernels);
     if (st != ZSAA_OK) return st;
   }
-  {
+  if (!fuse) {
     TRACE("advance", 0.0, 8.0);
     ZCK(launch_decode_advance(kc->step, s));
   }
@@ -2030,6 +2051,7 @@ zsaa_status zsaa_cache_create(zsaa_model* m, int B, int L, double accel, int max
   alloc(reinterpret_cast<void**>(&kc->rope_cos), static_cast<size_t>(n_pos) * (hd / 2) * sizeof(float));
   alloc(reinterpret_cast<void**>(&kc->rope_sin), static_cast<size_t>(n_pos) * (hd / 2) * sizeof(float));
   alloc(reinterpret_cast<void**>(&kc->qkv32), static_cast<size_t>(B) * m->ld_qkv * sizeof(float));
+  alloc(reinterpret_cast<void**>(&kc->norm_ss), 2 * static_cast<size_t>(c.d_model) * sizeof(float));
   alloc(reinterpret_cast<void**>(&kc->last_idx), static_cast<size_t>(B) * sizeof(int32_t));
   alloc(reinterpret_cast<void**>(&kc->step), sizeof(int));
   if (!ok) {
