@@ -178,13 +178,27 @@ __device__ __forceinline__ bool wait_flag(const int* f, int* status, volatile in
 
 __device__ __forceinline__ float silu_f(float g) { return g / (1.f + __expf(-g)); }
 
-__device__ __forceinline__ void store_bf16x16(bf16* dst, const float (&v)[16]) {
+// The epilogue's threads own a row each, so every access of a warp touches 32
+// lines and costs the load/store unit a pass over them: whole 32-byte sectors
+// per access (`wide`: base and row pitch allow them) halve the passes.  With the
+// RoPE tables shared by a tile's heads below, QKV at d 2048: 1100 rows 21.5 ->
+// 15.6 us, 6000 rows 58 -> 46; d 4096: 720 rows 30.8 -> 27.2; residual
+// projections 1-6% (d 4096, 3000 rows: 72.5 -> 68.5).
+__device__ __forceinline__ bool rows_wide(const void* base, int ld, int elem) {
+  return ((reinterpret_cast<uintptr_t>(base) | (static_cast<uintptr_t>(ld) * elem)) & 31) == 0;
+}
+
+__device__ __forceinline__ void store_bf16x16(bf16* dst, const float (&v)[16], bool wide) {
   uint32_t o[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) o[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
-  uint4* d = reinterpret_cast<uint4*>(dst);
-  d[0] = make_uint4(o[0], o[1], o[2], o[3]);
-  d[1] = make_uint4(o[4], o[5], o[6], o[7]);
+  if (wide) {
+    st_global_v8(dst, o);
+  } else {
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    d[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    d[1] = make_uint4(o[4], o[5], o[6], o[7]);
+  }
 }
 
 // Adds the fp32 partials of `count` contributors (slot c at ws + c * cstride,
@@ -233,6 +247,7 @@ __device__ __forceinline__ void fold_partials(uint32_t tbase, const float* ws, s
 template <int BN, int EPI>
 __device__ __forceinline__ void tile_epilogue(uint32_t tbase, int row, bool row_ok, int n0,
                                               const GemmParams& p) {
+  const bool wide = rows_wide(p.out, p.ldo, EPI == kEpiStoreF32 ? 4 : 2);
   if (EPI == kEpiSwiGLU) {
     bf16* out = static_cast<bf16*>(p.out);
     const int oc0 = n0 / 2;
@@ -252,7 +267,7 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tbase, int row, bool row_
         }
 #pragma unroll
         for (int e = 0; e < 16; ++e) v[e] = silu_f(gv[e]) * uv[e];
-        store_bf16x16(out + static_cast<size_t>(row) * p.ldo + oc0 + c, v);
+        store_bf16x16(out + static_cast<size_t>(row) * p.ldo + oc0 + c, v, wide);
       }
     }
   } else if (EPI == kEpiStoreF32) {
@@ -267,12 +282,16 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tbase, int row, bool row_
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (row_ok && n0 + c + 16 * h < p.N) {
-          float v[16];
+          float* dst = out + static_cast<size_t>(row) * p.ldo + n0 + c + 16 * h;
+          if (wide) {
+            st_global_v8(dst, r + 16 * h);
+            st_global_v8(dst + 8, r + 16 * h + 8);
+          } else {
 #pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[16 * h + e]);
-          float4* dst = reinterpret_cast<float4*>(out + static_cast<size_t>(row) * p.ldo + n0 + c + 16 * h);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            for (int q = 0; q < 4; ++q)
+              reinterpret_cast<uint4*>(dst)[q] =
+                  make_uint4(r[16 * h + 4 * q], r[16 * h + 4 * q + 1], r[16 * h + 4 * q + 2], r[16 * h + 4 * q + 3]);
+          }
         }
       }
     }
@@ -280,67 +299,64 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tbase, int row, bool row_
     bf16* out = static_cast<bf16*>(p.out);
     const int hd = p.hd, half = hd / 2;
     const int ps = row_ok ? p.pos[row] : 0;
+    // columns [0, rot) of the tile are rotated heads, the others value heads
+    const int rot = min(max(p.rope_cols - n0, 0), BN);
+    // A row's table entries serve every head: 16 of them are loaded and applied to all the tile's heads in turn.
+    // (Loaded per head they were most of the epilogue's memory accesses.)
+    float cs[16], sn[16];
+    const float* ct = p.cos_t + static_cast<size_t>(ps) * half;
+    const float* st = p.sin_t + static_cast<size_t>(ps) * half;
+    bf16* orow = out + static_cast<size_t>(row) * p.ldo + n0;
 #pragma unroll 1
-    for (int hs = 0; hs < BN; hs += hd) {
-      const bool rot = n0 + hs < p.rope_cols;
-      float vss = 0.f;  // value heads: sum of squares of the stored (bf16) values
-#pragma unroll 1
-      for (int c = 0; c < half; c += 16) {
-        uint32_t x1[16], x2[16];
-        float4 cs4[4], sn4[4];
-        if (rot && row_ok) {  // table loads first: their latency overlaps the TMEM load
-          const float4* cp = reinterpret_cast<const float4*>(p.cos_t + static_cast<size_t>(ps) * half + c);
-          const float4* sp = reinterpret_cast<const float4*>(p.sin_t + static_cast<size_t>(ps) * half + c);
+    for (int c = 0; c < half && rot > 0; c += 16) {
+      if (row_ok) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            cs4[q] = __ldg(cp + q);
-            sn4[q] = __ldg(sp + q);
-          }
+        for (int q = 0; q < 16; q += 8) {
+          ld_global_v8(reinterpret_cast<uint32_t*>(cs + q), ct + c + q);
+          ld_global_v8(reinterpret_cast<uint32_t*>(sn + q), st + c + q);
         }
+      }
+#pragma unroll 1
+      for (int hs = 0; hs < rot; hs += hd) {
+        uint32_t x1[16], x2[16];
         __syncwarp();
         tmem_ld16(tbase + hs + c, x1);
         tmem_ld16(tbase + hs + half + c, x2);
         tmem_ld_wait();
         if (row_ok && n0 + hs < p.N) {
-          float a1[16], a2[16], y1[16], y2[16];
+          float y1[16], y2[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
-            a1[e] = __uint_as_float(x1[e]);
-            a2[e] = __uint_as_float(x2[e]);
+            const float a = __uint_as_float(x1[e]), b = __uint_as_float(x2[e]);
+            y1[e] = a * cs[e] - b * sn[e];
+            y2[e] = b * cs[e] + a * sn[e];
           }
-          if (rot) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float4 cs = cs4[q], sn = sn4[q];
-              const float cv[4] = {cs.x, cs.y, cs.z, cs.w}, sv[4] = {sn.x, sn.y, sn.z, sn.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float a = a1[4 * q + e], b = a2[4 * q + e];
-                y1[4 * q + e] = a * cv[e] - b * sv[e];
-                y2[4 * q + e] = b * cv[e] + a * sv[e];
-              }
-            }
-          } else {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              y1[e] = a1[e];
-              y2[e] = a2[e];
-            }
-          }
-          bf16* rowp = out + static_cast<size_t>(row) * p.ldo + n0 + hs;
-          store_bf16x16(rowp + c, y1);
-          store_bf16x16(rowp + half + c, y2);
-          if (!rot && p.vnorm_out != nullptr) {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const float r1 = __bfloat162float(__float2bfloat16_rn(y1[e]));
-              const float r2 = __bfloat162float(__float2bfloat16_rn(y2[e]));
-              vss += r1 * r1 + r2 * r2;
-            }
-          }
+          store_bf16x16(orow + hs + c, y1, wide);
+          store_bf16x16(orow + hs + half + c, y2, wide);
         }
       }
-      if (!rot && p.vnorm_out != nullptr && row_ok && n0 + hs < p.N) {
+    }
+#pragma unroll 1
+    for (int hs = rot; hs < BN; hs += hd) {
+      float vss = 0.f;  // sum of squares of the stored (bf16) values
+#pragma unroll 1
+      for (int c = 0; c < hd; c += 16) {
+        uint32_t x[16];
+        __syncwarp();
+        tmem_ld16(tbase + hs + c, x);
+        tmem_ld_wait();
+        if (row_ok && n0 + hs < p.N) {
+          float y[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            y[e] = __uint_as_float(x[e]);
+            const float r = __bfloat162float(__float2bfloat16_rn(y[e]));
+            vss += r * r;
+          }
+          store_bf16x16(orow + hs + c, y, wide);
+        }
+      }
+      if (p.vnorm_out != nullptr && row_ok && n0 + hs < p.N) {
         const int groups = (p.N - p.rope_cols) / hd;
         p.vnorm_out[static_cast<size_t>(row) * groups + (n0 + hs - p.rope_cols) / hd] = sqrtf(vss);
       }
@@ -349,23 +365,31 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tbase, int row, bool row_
     bf16* out = static_cast<bf16*>(p.out);
     const bf16* res = static_cast<const bf16*>(p.resid);
     const size_t rowoff = static_cast<size_t>(row) * p.ldo + n0;
-    uint4 rc[4], rn[4];
-    auto load_res = [&](int c, uint4 (&r)[4]) {
+    // residual of 32 columns, requested one chunk ahead of their use (two ahead was slower)
+    uint32_t rc[16], rn[16];
+    const bool wide_res = EPI == kEpiResid && rows_wide(p.resid, p.ldo, 2);
+    auto load_res = [&](int c, uint32_t (&r)[16]) {
+      if (EPI != kEpiResid) return;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (EPI == kEpiResid && row_ok && n0 + c + 16 * h < p.N) {
-          const uint4* rp = reinterpret_cast<const uint4*>(res + rowoff + c + 16 * h);
-          r[2 * h] = rp[0];
-          r[2 * h + 1] = rp[1];
-        } else {
-          r[2 * h] = r[2 * h + 1] = make_uint4(0u, 0u, 0u, 0u);
+        if (row_ok && c < BN && n0 + c + 16 * h < p.N) {
+          const bf16* src = res + rowoff + c + 16 * h;
+          if (wide_res) {
+            ld_global_v8(r + 8 * h, src);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const uint4 u = reinterpret_cast<const uint4*>(src)[q];
+              r[8 * h + 4 * q] = u.x, r[8 * h + 4 * q + 1] = u.y, r[8 * h + 4 * q + 2] = u.z, r[8 * h + 4 * q + 3] = u.w;
+            }
+          }
         }
       }
     };
     load_res(0, rc);
 #pragma unroll 1
     for (int c = 0; c < BN; c += 32) {
-      if (c + 32 < BN) load_res(c + 32, rn);  // in flight while this chunk drains TMEM
+      load_res(c + 32, rn);
       uint32_t r[32];
       __syncwarp();
       tmem_ld16(tbase + c, *reinterpret_cast<uint32_t(*)[16]>(r));
@@ -378,19 +402,19 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tbase, int row, bool row_
 #pragma unroll
           for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[16 * h + e]);
           if (EPI == kEpiResid) {
-            const uint32_t rr[8] = {rc[2 * h].x, rc[2 * h].y, rc[2 * h].z, rc[2 * h].w,
-                                    rc[2 * h + 1].x, rc[2 * h + 1].y, rc[2 * h + 1].z, rc[2 * h + 1].w};
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              v[2 * e] += bf16lo(rr[e]);
-              v[2 * e + 1] += bf16hi(rr[e]);
+              v[2 * e] += bf16lo(rc[8 * h + e]);
+              v[2 * e + 1] += bf16hi(rc[8 * h + e]);
             }
           }
-          store_bf16x16(out + rowoff + c + 16 * h, v);
+          store_bf16x16(out + rowoff + c + 16 * h, v, wide);
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) rc[q] = rn[q];
+      for (int q = 0; q < 16; ++q) {
+        rc[q] = rn[q];
+      }
     }
   }
 }
