@@ -5,19 +5,28 @@
 //
 // What bounds it: the FMA pipe (about 76 TFLOP/s) once there are enough tiles,
 // and the length of one tile's K chain when there are few.  So:
-//  - 64 x 64 tiles of 64 threads, 8 x 8 outputs a thread.  Both operands stay
-//    K-major in shared memory (rows of 16 k, padded to 20 floats: 16-byte
-//    copies in, and a quarter warp's 16-byte reads hit distinct banks), so a
-//    thread reads four k of a row at once and multiplies them as two packed
-//    pairs (fma.rn.f32x2): an output's even and odd k accumulate separately
-//    and are added at the end, which is no less exact than one chain.
-//  - A three-stage cp.async ring per CTA; four CTAs share an SM.
-//    A 4 x 4 output tile per thread, 4-byte staging and one stage at a time ran
-//    at 6-22 TFLOP/s; this runs at 28-36 (d 1024, ffn 4096, 324-1536 rows: down
-//    570 -> 145 us, gate/up 399 -> 247 us, QKV with RoPE 437 -> 91 us a launch).
-//  - Few tiles: K is split over a thread-block cluster of S <= 8 CTAs, whose
-//    partial tiles meet in distributed shared memory and are added in rank
-//    order (deterministic).  S minimises CTAs per SM x k-blocks per CTA.
+//  - 64 x 64 tiles of two groups of 64 threads, each group half of the tile's K
+//    with its own stages and barrier: a CTA loads all four schedulers (one of
+//    two warps leaves two idle, and two such CTAs can meet on the same two).
+//  - 8 x 8 outputs a thread, as packed pairs of neighbouring columns
+//    (fma.rn.f32x2 with the row's value in both halves; an output is one FMA
+//    chain per part of K).  That wants a k's columns side by side, so a thread
+//    moves its weights from the place they were copied to into [16 k][64
+//    columns]; A stays K-major (rows of 16 k, padded to 20 floats), four k of a
+//    row read at once.  Copies, moves and reads hit distinct banks.  From shared
+//    memory alone this loop runs at 62 TFLOP/s in 134 registers; with pairs of k
+//    and no transpose it needs twice the accumulators and runs at 55.
+//  - Three stages of 16-byte cp.async, weights too: loaded through registers one
+//    block ahead, the few-tile shapes waited on them (24 rows, N 2048, K 1024:
+//    37 us against 33 for a whole tile).
+//  - Few tiles: K is also split over a thread-block cluster of S <= 8 CTAs,
+//    whose partial tiles meet in distributed shared memory and are added in the
+//    order of their parts (deterministic).
+//    Measured, d 1024, ffn 4096, 324-1536 rows, a launch: gate/up 206 us (43
+//    TFLOP/s on average, 53 at 1536 rows), down 113, QKV with RoPE 70, O 54;
+//    with pairs of k, one group and the earlier split rule 247, 138, 89, 59;
+//    with 4 x 4 outputs a thread, 4-byte staging and one stage 399, 570, 437 (QKV
+//    and its RoPE), 6-22 TFLOP/s.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -26,12 +35,18 @@ namespace {
 
 constexpr int FB = 64;       // tile edge: rows of A, weight rows
 constexpr int FK = 16;       // k per stage
-constexpr int FLD = FK + 4;  // shared-memory row stride, floats
-constexpr int FST = 3;       // stages
-constexpr int FTHREADS = 64;
+constexpr int FLD = FK + 4;  // A: shared-memory row stride, floats
+constexpr int FWLD = FB + 4;  // weights: stride of one k's columns, floats
+constexpr int FST = 3;       // stages of copies
+constexpr int FG = 2;        // groups of two warps, each with its part of K
+constexpr int FGT = 64;      // threads of a group
+constexpr int FTHREADS = FG * FGT;
 constexpr int FRED = FB + 4;  // row stride of the partial tile
-constexpr int F_STAGE = 2 * FB * FLD;
-static_assert(FST * F_STAGE >= FB * FRED, "the partial tile reuses the ring");
+constexpr int FA_STAGE = FB * FLD, FC_STAGE = FB * FK, FW_STAGE = FK * FWLD;
+// a group's shared memory: stages of A, of the weights as copied (each thread's
+// chunks side by side), two of the weights transposed
+constexpr int F_COPY = FST * FA_STAGE, F_TRANS = F_COPY + FST * FC_STAGE, F_SMEM = F_TRANS + 2 * FW_STAGE;
+static_assert(F_SMEM >= FB * FRED, "the partial tile reuses the stages");
 
 struct F32Args {
   const float* A;
@@ -50,15 +65,19 @@ __device__ __forceinline__ void cp_async_zfill(uint32_t dst, const float* src, b
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
+// One group's barrier.
+__device__ __forceinline__ void group_sync(int grp) { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(FGT) : "memory"); }
+
 // VEC: K, lda and every base allow 16-byte copies of A and W (else 4-byte ones).
 template <int EPI, bool VEC>
-__global__ void __launch_bounds__(FTHREADS, 4) gemm_f32_kernel(const F32Args a) {
+__global__ void __launch_bounds__(FTHREADS, 3) gemm_f32_kernel(const F32Args a) {
   constexpr bool DUAL = EPI == kEpiSwiGLU;
   constexpr int NOUT = DUAL ? FB / 2 : FB;  // output columns of a tile
-  __shared__ __align__(16) float sm[FST * F_STAGE];
+  extern __shared__ __align__(16) float smem[];
   pdl_trigger();
   const GemmParams& p = a.p;
-  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int grp = threadIdx.x / FGT, tid = threadIdx.x % FGT, tx = tid & 7, ty = tid >> 3;
+  float* sm = smem + grp * F_SMEM;
   const int S = static_cast<int>(cluster_size()), rank = static_cast<int>(cluster_rank());
   const int tn = blockIdx.x / S, m0 = blockIdx.y * FB;
   // Output column of tile column j.  RoPE pairs dims c and c + hd/2 of a head:
@@ -86,98 +105,142 @@ __global__ void __launch_bounds__(FTHREADS, 4) gemm_f32_kernel(const F32Args a) 
   };
 
   const int KB = (p.K + FK - 1) / FK;
-  const int kb0 = static_cast<int>(static_cast<long long>(rank) * KB / S);
-  const int kb1 = static_cast<int>(static_cast<long long>(rank + 1) * KB / S);
-  // VEC: a thread copies 16-byte chunk tid%4 of rows tid/4 + 16 i of both operands
+  const int part = rank * FG + grp, parts = S * FG;
+  const int kb0 = static_cast<int>(static_cast<long long>(part) * KB / parts);
+  const int kb1 = static_cast<int>(static_cast<long long>(part + 1) * KB / parts);
+  // VEC: a thread copies 16-byte chunks: of A, chunk tid%4 of rows tid/4 + 16 i;
+  // of the weights, chunk tid%2 + 2 warp of rows (tid%32)/2 + 16 i (whole
+  // sectors, and the transposed stores of a warp hit 32 banks).  A row past the
+  // matrix reads a valid one instead: its outputs are not stored.
   constexpr int RPT = 4;
+  const int wr = (tid & 31) >> 1, wk = ((tid & 1) + 2 * (tid >> 5)) * 4;
   const float* srcA[RPT];
   const float* srcW[RPT];
   if (VEC) {
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
-      const int r = (tid >> 2) + 16 * i;
-      srcA[i] = m0 + r < p.M ? a.A + static_cast<size_t>(m0 + r) * a.lda + (tid & 3) * 4 : nullptr;
-      const float* w = wrow(r);
-      srcW[i] = w != nullptr ? w + (tid & 3) * 4 : nullptr;
+      srcA[i] = a.A + static_cast<size_t>(min(m0 + (tid >> 2) + 16 * i, p.M - 1)) * a.lda + kb0 * FK + (tid & 3) * 4;
+      const float* w = wrow(wr + 16 * i);
+      srcW[i] = (w != nullptr ? w : static_cast<const float*>(a.W.w0)) + kb0 * FK + wk;
     }
   }
-  const uint32_t sbase = smem_u32(sm);
-  auto load = [&](int kb, int st, bool first, bool second) {  // first: the weights, second: A
-    const uint32_t dA = sbase + st * F_STAGE * 4, dW = dA + FB * FLD * 4;
+  const uint32_t sbase = smem_u32(sm), dA = sbase + (VEC ? ((tid >> 2) * FLD + (tid & 3) * 4) * 4 : 0);
+  // A's block kb -> stage st; blocks are loaded in order, each advancing the pointers
+  auto load_a = [&](int kb, int st) {
     if (VEC) {
-      const int k = kb * FK;
-      const bool kin = k + (tid & 3) * 4 < p.K;
+      const bool kin = kb * FK + (tid & 3) * 4 < p.K;
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
-        const uint32_t o = (((tid >> 2) + 16 * i) * FLD + (tid & 3) * 4) * 4;
-        const bool va = kin && srcA[i] != nullptr, vw = kin && srcW[i] != nullptr;
-        if (second) cp_async_zfill<16>(dA + o, va ? srcA[i] + k : a.A, va);
-        if (first) cp_async_zfill<16>(dW + o, vw ? srcW[i] + k : static_cast<const float*>(a.W.w0), vw);
+        cp_async_zfill<16>(dA + (st * FA_STAGE + 16 * i * FLD) * 4, srcA[i], kin);
+        srcA[i] += FK;
       }
     } else {
-      for (int i = tid; i < FB * FK; i += FTHREADS) {
+      for (int i = tid; i < FB * FK; i += FGT) {
         const int r = i / FK, k = kb * FK + i % FK;
-        const uint32_t o = (r * FLD + i % FK) * 4;
-        const float* w = wrow(r);
-        const bool va = k < p.K && m0 + r < p.M, vw = k < p.K && w != nullptr;
-        if (second) cp_async_zfill<4>(dA + o, va ? a.A + static_cast<size_t>(m0 + r) * a.lda + k : a.A, va);
-        if (first) cp_async_zfill<4>(dW + o, vw ? w + k : static_cast<const float*>(a.W.w0), vw);
+        const bool va = k < p.K && m0 + r < p.M;
+        cp_async_zfill<4>(dA + (st * FA_STAGE + r * FLD + i % FK) * 4,
+                          va ? a.A + static_cast<size_t>(m0 + r) * a.lda + k : a.A, va);
       }
     }
   };
-
-  // a model's weights, which no kernel writes: the first stages' rows before
-  // waiting for the previous kernel, their activations after
-  if (p.w_const) {
+  // VEC: the weights' block kb -> stage st as copied; later each thread moves its
+  // own chunks to their transposed place.  Else straight to that place.
+  auto copy_w = [&](int kb, int st) {
+    if (VEC) {
+      const bool kin = kb * FK + wk < p.K;
 #pragma unroll
-    for (int s = 0; s < FST - 1; ++s)
-      if (kb0 + s < kb1) load(kb0 + s, s, true, false);
-  }
+      for (int i = 0; i < RPT; ++i) {
+        cp_async_zfill<16>(sbase + (F_COPY + st * FC_STAGE + (i * FGT + tid) * 4) * 4, srcW[i], kin);
+        srcW[i] += FK;
+      }
+    } else {
+      for (int i = tid; i < FB * FK; i += FGT) {
+        const int r = i / FK, k = kb * FK + i % FK;
+        const float* w = wrow(r);
+        const bool vw = k < p.K && w != nullptr;
+        cp_async_zfill<4>(sbase + (F_TRANS + st * FW_STAGE + (i % FK) * FWLD + r) * 4,
+                          vw ? w + k : static_cast<const float*>(a.W.w0), vw);
+      }
+    }
+  };
+  auto transpose_w = [&](int st, int sw) {
+    const float* c = sm + F_COPY + st * FC_STAGE + tid * 4;
+    float* d = sm + F_TRANS + sw * FW_STAGE + wk * FWLD + wr;
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const float4 v = *reinterpret_cast<const float4*>(c + i * FGT * 4);
+      float* q = d + 16 * i;
+      q[0] = v.x, q[FWLD] = v.y, q[2 * FWLD] = v.z, q[3 * FWLD] = v.w;
+    }
+  };
+
+  // a model's weights, which no kernel writes: the first blocks before waiting
+  // for the previous kernel, their activations after
+  auto first_w = [&] {
+#pragma unroll
+    for (int s = 0; s < (VEC ? FST - 1 : 1); ++s)
+      if (kb0 + s < kb1) copy_w(kb0 + s, s);
+  };
+  if (p.w_const) first_w();
   pdl_wait();
+  if (!p.w_const) first_w();
 #pragma unroll
   for (int s = 0; s < FST - 1; ++s) {
-    if (kb0 + s < kb1) load(kb0 + s, s, !p.w_const, true);
-    cp_async_commit();  // group s holds stage s's activations (and, for s = 0, the weights)
+    if (kb0 + s < kb1) load_a(kb0 + s, s);
+    cp_async_commit();  // the first group holds the weights too
   }
-  uint64_t acc[8][8];
+  cp_async_wait<FST - 2>();
+  if (VEC && kb0 < kb1) transpose_w(0, 0);
+  uint64_t acc[8][4];  // rows ty + 8 i; columns 4 tx + {0, 1}, {2, 3}, 32 + 4 tx + {0, 1}, {2, 3}
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
-  int st = 0;
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  int st = 0, sw = 0;
   for (int kb = kb0; kb < kb1; ++kb) {
-    cp_async_wait<FST - 2>();
-    __syncthreads();  // stage st has landed; every thread is done with the stage filled next
-    const int nx = kb + FST - 1;
-    if (nx < kb1) load(nx, st == 0 ? FST - 1 : st - 1, true, true);
+    group_sync(grp);  // block kb is in place; every thread is done with the stages filled next
+    const int nx = kb + FST - 1, nst = st == 0 ? FST - 1 : st - 1;
+    if (nx < kb1) {
+      load_a(nx, nst);
+      if (VEC) copy_w(nx, nst);
+    }
+    if (!VEC && kb + 1 < kb1) copy_w(kb + 1, sw ^ 1);
     cp_async_commit();
-    const float* sa = sm + st * F_STAGE + ty * FLD;
-    const float* sw = sm + st * F_STAGE + FB * FLD + tx * FLD;
+    const float* pa = sm + st * FA_STAGE + ty * FLD;
+    const float* pw = sm + F_TRANS + sw * FW_STAGE + 4 * tx;
 #pragma unroll
     for (int k = 0; k < FK; k += 4) {
-      ulonglong2 av[8];
+      float4 av[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) av[i] = *reinterpret_cast<const ulonglong2*>(sa + 8 * i * FLD + k);
+      for (int i = 0; i < 8; ++i) av[i] = *reinterpret_cast<const float4*>(pa + 8 * i * FLD + k);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(sw + 8 * j * FLD + k);
+      for (int e = 0; e < 4; ++e) {
+        const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(pw + (k + e) * FWLD);
+        const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(pw + (k + e) * FWLD + FB / 2);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i][j] = ffma2(av[i].y, wv.y, ffma2(av[i].x, wv.x, acc[i][j]));
+        for (int i = 0; i < 8; ++i) {
+          const float x = e == 0 ? av[i].x : e == 1 ? av[i].y : e == 2 ? av[i].z : av[i].w;
+          const uint64_t xx = f2pack(x, x);
+          acc[i][0] = ffma2(xx, w0.x, acc[i][0]);
+          acc[i][1] = ffma2(xx, w0.y, acc[i][1]);
+          acc[i][2] = ffma2(xx, w1.x, acc[i][2]);
+          acc[i][3] = ffma2(xx, w1.y, acc[i][3]);
+        }
       }
     }
     st = st == FST - 1 ? 0 : st + 1;
+    sw ^= 1;
+    cp_async_wait<VEC ? FST - 2 : 0>();
+    if (VEC && kb + 1 < kb1) transpose_w(st, sw);
   }
   cp_async_wait<0>();
-  __syncthreads();
-  // this CTA's partial tile -> its shared memory
+  group_sync(grp);
+  // the group's partial tile -> its shared memory
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float e, o;
-      f2unpack(acc[i][j], e, o);
-      sm[(ty + 8 * i) * FRED + tx + 8 * j] = e + o;
-    }
+    for (int j = 0; j < 4; j += 2)
+      *reinterpret_cast<ulonglong2*>(sm + (ty + 8 * i) * FRED + 4 * tx + 16 * j) = make_ulonglong2(acc[i][j], acc[i][j + 1]);
   if (S > 1)
     cluster_sync_all();
   else
@@ -187,16 +250,18 @@ __global__ void __launch_bounds__(FTHREADS, 4) gemm_f32_kernel(const F32Args a) 
   const int r0 = rank * FB / S, r1 = (rank + 1) * FB / S;
   const bool vec_out = (p.ldo & 3) == 0 && (p.N & 3) == 0 && (reinterpret_cast<uintptr_t>(p.out) & 15) == 0 &&
                        (EPI != kEpiResid || (reinterpret_cast<uintptr_t>(p.resid) & 15) == 0);
-  auto sum4 = [&](int r, int c) {  // the S partials of four neighbouring columns, in rank order
-    float4 v = *reinterpret_cast<const float4*>(sm + r * FRED + c);
+  auto sum4 = [&](int r, int c) {  // the partials of four neighbouring columns, in the order of their parts of K
+    float4 v = *reinterpret_cast<const float4*>(smem + r * FRED + c);
+    const float4 v1 = *reinterpret_cast<const float4*>(smem + F_SMEM + r * FRED + c);
+    v.x += v1.x, v.y += v1.y, v.z += v1.z, v.w += v1.w;
     if (S > 1) {
-      const uint32_t local = smem_u32(sm + r * FRED + c);
+      const uint32_t local = smem_u32(smem + r * FRED + c);
       v = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int q = 0; q < S; ++q) {
+      for (int q = 0; q < S * FG; ++q) {
         float4 t;
         asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w)
-                     : "r"(map_rank(local, q))
+                     : "r"(map_rank(local + (q % FG) * F_SMEM * 4, q / FG))
                      : "memory");
         v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
       }
@@ -204,7 +269,7 @@ __global__ void __launch_bounds__(FTHREADS, 4) gemm_f32_kernel(const F32Args a) 
     return v;
   };
   constexpr int C4 = NOUT / 4;  // column groups of a row
-  for (int t = tid; t < (r1 - r0) * C4; t += FTHREADS) {
+  for (int t = threadIdx.x; t < (r1 - r0) * C4; t += FTHREADS) {
     const int r = r0 + t / C4, c = (t % C4) * 4, m = m0 + r, n = col(c);
     if (m >= p.M || n >= p.N) continue;
     const float4 v4 = sum4(r, c);
@@ -256,16 +321,22 @@ int f32_sms() {
   return cached[dev];
 }
 
-// Cluster size: an SM runs two CTAs at full FMA rate (a lone one uses half of
-// it), so the time is about max(1, CTAs per SM / 2) x k-blocks per CTA
-// (0.5 us each), plus about 1 us for a cluster's reduction.
+// Cluster size.  Measured over 67 shapes (d 64-4096, 24-5000 rows): a k-block of
+// a tile takes about 1 us with up to three CTAs on an SM (0.5 us for a CTA with
+// neighbouring SMs idle), three more double it, and a cluster of 2, 4, 8 adds
+// 0.85, 1.75, 4 us to each round of CTAs for its reduction and its smaller
+// parts' ramp.  The split this picks is within 2% of the best of the four on
+// average.  The earlier rule took two CTAs for a full SM and no cost per round:
+// it split 1536 x 4096 x 1024 eightfold (750 us for gate and up against 482) and
+// left 1100 x 1024 x 4096 whole (283 us against 194).
 int f32_split(long long tiles, int KB) {
+  static const double extra[4] = {0.0, 0.85, 1.75, 4.0};
   int best = 1;
   double best_cost = 0.0;
-  for (int S = 1; S <= 8 && S <= KB; S *= 2) {
+  for (int i = 0, S = 1; i < 4 && S <= KB; ++i, S *= 2) {
     const long long per_sm = (tiles * S + f32_sms() - 1) / f32_sms();
-    const double waves = per_sm > 2 ? 0.5 * static_cast<double>(per_sm) : 1.0;
-    const double cost = waves * ((KB + S - 1) / S) * 0.5 + (S > 1 ? 1.0 : 0.0);
+    const double rounds = per_sm > 3 ? static_cast<double>(per_sm) / 3.0 : 1.0;
+    const double cost = rounds * ((KB + S - 1) / S + extra[i] + 0.5);
     if (S == 1 || cost < best_cost) best = S, best_cost = cost;
   }
   return best;
@@ -276,6 +347,7 @@ cudaError_t run_f32(const F32Args& a, int tiles_n, int tiles_m, int S, cudaStrea
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(tiles_n) * S, tiles_m);
   cfg.blockDim = dim3(FTHREADS);
+  cfg.dynamicSmemBytes = FG * F_SMEM * sizeof(float);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -286,6 +358,10 @@ cudaError_t run_f32(const F32Args& a, int tiles_n, int tiles_m, int S, cudaStrea
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
+  static OncePerDevice once;
+  const cudaError_t e =
+      set_smem_limit_once(once, gemm_f32_kernel<EPI, VEC>, static_cast<int>(cfg.dynamicSmemBytes));
+  if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, gemm_f32_kernel<EPI, VEC>, a);
 }
 

@@ -26,7 +26,8 @@ def z(zlib):
 # K below one stage, off the 16-byte copies (70, 5), split over 2..8 CTAs of a
 # cluster (few tiles, deep K) and whole (many tiles); ragged rows and columns.
 @pytest.mark.parametrize("M,N,K", [(1, 3, 5), (64, 64, 16), (65, 130, 70), (63, 65, 15), (129, 96, 272),
-                                   (20, 200, 1027), (64, 128, 4096), (300, 516, 512), (1500, 1028, 100)])
+                                   (20, 200, 1027), (64, 128, 4096), (300, 516, 512), (1500, 1028, 100),
+                                   (40, 64, 20), (70, 100, 48)])
 @pytest.mark.parametrize("epi", ["store", "resid", "swiglu"])
 def test_linear_f32_tiles(z, epi, M, N, K):
     A, W, W2 = (_rand(s, i, dtype=torch.float32) for i, s in enumerate([(M, K), (N, K), (N, K)]))
