@@ -126,14 +126,16 @@ inline FastDiv fast_div(int d) {
 
 // Variable-length batches keep the rows of B sequences packed, sequence b at
 // rows [cu[b], cu[b+1]) (cu[0] = 0, strictly increasing).  Sequence of row r:
+// A whole warp, with the same r, probes 32 places at a time.
 __device__ __forceinline__ int seq_of_row(const int* __restrict__ cu, int B, int r) {
-  int lo = 0, hi = B;  // cu[lo] <= r < cu[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(cu + mid) <= r)
-      lo = mid;
-    else
-      hi = mid;
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = B;  // cu[lo] <= r < cu[lo + n]
+  while (n > 1) {
+    const int step = (n + 31) >> 5, i = lane * step;
+    const unsigned le = __ballot_sync(0xffffffffu, i < n && __ldg(cu + lo + i) <= r);
+    const int at = (__popc(le) - 1) * step;  // place 0 always counts
+    lo += at;
+    n = min(step, n - at);
   }
   return lo;
 }

@@ -1,7 +1,10 @@
 // Row-wise kernels of the pruned prefill: embedding gather, RMSNorm, row-norm
 // scores of the isolated path (Sec. 3.3 with unit column mass), per-sequence
-// top-k selection, row compaction, fp32 RoPE and the classifier head.  All are HBM-bound: one warp per row, 16-byte
-// vector accesses, fp32 arithmetic.
+// top-k selection, row compaction, fp32 RoPE and the classifier head.  One warp
+// per row, 16-byte vector accesses, fp32 arithmetic.
+#include <algorithm>
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -15,6 +18,40 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kMaxVecPerLane = 16;
 
 inline int row_blocks(int rows) { return (rows + kWarpsPerBlock - 1) / kWarpsPerBlock; }
+
+// The kernels that norm whole rows keep Q vectors of a row per lane, and as many
+// blocks as stay resident walk the rows.  They are bound by HBM for many rows
+// and by the chain weights -> index -> row -> sum -> store for few.  One size of
+// 16 vectors for every row length held 95 registers, so 16 warps an SM, and each
+// block staged the norm weights for eight rows only: embedding and norm of 16384
+// rows of 2048 took 61 us with events (3.3 TB/s), compaction and norm 20 us on
+// average over a forward; Q by the row length and a row loop 36 us (5.6 TB/s) and
+// 13 us.
+__host__ __device__ constexpr int norm_blocks_per_sm(int Q) { return Q >= 16 ? 2 : Q >= 8 ? 4 : 6; }
+
+inline int norm_grid(int rows, int Q) {
+  static int cached[64] = {};
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    if (cached[dev] == 0 &&
+        (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0))
+      sms = 148;
+    if (cached[dev] == 0) cached[dev] = sms;
+    sms = cached[dev];
+  }
+  return std::min(row_blocks(rows), sms * norm_blocks_per_sm(Q));
+}
+
+// fn(std::integral_constant<int, Q>) for the smallest Q that holds vec vectors: a
+// larger one costs registers (resident warps) and predicated-off instructions
+template <class Fn>
+cudaError_t norm_dispatch(int vec, Fn&& fn) {
+  if (vec <= 64) return fn(std::integral_constant<int, 2>());
+  if (vec <= 128) return fn(std::integral_constant<int, 4>());
+  if (vec <= 256) return fn(std::integral_constant<int, 8>());
+  return fn(std::integral_constant<int, kMaxVecPerLane>());
+}
+
 
 // ---------------------------------------------------------------- embedding
 
@@ -80,32 +117,13 @@ __device__ __forceinline__ void stage_norm_weights(const uint4* __restrict__ w, 
   __syncthreads();
 }
 
-// bf16 rows of at most 32 * kMaxVecPerLane vectors: one warp per row, the row
-// loaded into registers once (every load of a lane in flight together), its
-// sum of squares, then x = h / rms * w with the weights from shared memory.
-__global__ void rmsnorm_bf16_reg_kernel(const uint4* __restrict__ h, const uint4* __restrict__ w,
-                                        int rows, int vec, float eps, uint4* __restrict__ x) {
-  extern __shared__ uint4 sw[];
-  pdl_trigger();
-  stage_norm_weights(w, vec, sw);
-  pdl_wait();
-  h = after_wait(h);
-  const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (r >= rows) return;
-  const uint4* hr = h + static_cast<size_t>(r) * vec;
-  uint4* xr = x + static_cast<size_t>(r) * vec;
-  uint4 u[kMaxVecPerLane];
+// 1/rms of a row held as Q vectors a lane (lane's vector q: lane + 32 q).
+template <int Q>
+__device__ __forceinline__ float row_inv_rms(const uint4 (&u)[Q], int lane, int vec, float eps) {
   float ss = 0.f;
 #pragma unroll
-  for (int q = 0; q < kMaxVecPerLane; ++q) {
-    const int v = lane + 32 * q;
-    if (v < vec) u[q] = hr[v];
-  }
-#pragma unroll
-  for (int q = 0; q < kMaxVecPerLane; ++q) {
-    const int v = lane + 32 * q;
-    if (v < vec) {
+  for (int q = 0; q < Q; ++q) {
+    if (lane + 32 * q < vec) {
       const uint32_t e4[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -115,9 +133,15 @@ __global__ void rmsnorm_bf16_reg_kernel(const uint4* __restrict__ h, const uint4
     }
   }
   ss = warp_sum(ss);
-  const float inv = rsqrtf(ss / static_cast<float>(vec * 8) + eps);
+  return rsqrtf(ss / static_cast<float>(vec * 8) + eps);
+}
+
+// x = h * inv * w of such a row, the weights in shared memory
+template <int Q>
+__device__ __forceinline__ void write_normed(const uint4 (&u)[Q], float inv, const uint4* sw, int lane, int vec,
+                                             uint4* __restrict__ xr) {
 #pragma unroll
-  for (int q = 0; q < kMaxVecPerLane; ++q) {
+  for (int q = 0; q < Q; ++q) {
     const int v = lane + 32 * q;
     if (v < vec) {
       const uint4 wv = sw[v];
@@ -129,6 +153,30 @@ __global__ void rmsnorm_bf16_reg_kernel(const uint4* __restrict__ h, const uint4
         o[e] = pack_bf16x2(bf16lo(e4[e]) * inv * bf16lo(w4[e]), bf16hi(e4[e]) * inv * bf16hi(w4[e]));
       xr[v] = make_uint4(o[0], o[1], o[2], o[3]);
     }
+  }
+}
+
+// bf16 rows of at most 32 Q vectors: one warp per row, the row loaded into
+// registers once (every load of a lane in flight together), its sum of
+// squares, then x = h / rms * w with the weights from shared memory.
+template <int Q>
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, norm_blocks_per_sm(Q))
+    rmsnorm_bf16_reg_kernel(const uint4* __restrict__ h, const uint4* __restrict__ w, int rows, int vec, float eps,
+                            uint4* __restrict__ x) {
+  extern __shared__ uint4 sw[];
+  pdl_trigger();
+  stage_norm_weights(w, vec, sw);
+  pdl_wait();
+  h = after_wait(h);
+  const int lane = threadIdx.x & 31, stride = gridDim.x * kWarpsPerBlock;
+  for (int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); r < rows; r += stride) {
+    const uint4* hr = h + static_cast<size_t>(r) * vec;
+    uint4 u[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (lane + 32 * q < vec) u[q] = hr[lane + 32 * q];
+    const float inv = row_inv_rms<Q>(u, lane, vec, eps);
+    write_normed<Q>(u, inv, sw, lane, vec, x + static_cast<size_t>(r) * vec);
   }
 }
 
@@ -515,91 +563,56 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ src, int N, int k, 
 //     pos_in[that row] -- the kept rows of the previous layer, already normed
 //     for the next layer's attention.
 // An index outside its range sets kStatusBadIndex and copies row 0.
-__global__ void rows_norm_bf16_kernel(const uint4* __restrict__ src, const int32_t* __restrict__ tok,
-                                      int vocab, int L, const int32_t* __restrict__ idx, int N,
-                                      int k, const int32_t* __restrict__ pos_in, int rows, int vec,
-                                      const uint4* __restrict__ w, float eps,
-                                      uint4* __restrict__ h_out, uint4* __restrict__ x_out,
-                                      int32_t* __restrict__ pos_out, int* status,
-                                      const int* __restrict__ cu_src, const int* __restrict__ cu_dst,
-                                      int nseq) {
+template <int Q>
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, norm_blocks_per_sm(Q))
+    rows_norm_bf16_kernel(const uint4* __restrict__ src, const int32_t* __restrict__ tok, int vocab, int L,
+                          const int32_t* __restrict__ idx, int N, int k, const int32_t* __restrict__ pos_in, int rows,
+                          int vec, const uint4* __restrict__ w, float eps, uint4* __restrict__ h_out,
+                          uint4* __restrict__ x_out, int32_t* __restrict__ pos_out, int* status,
+                          const int* __restrict__ cu_src, const int* __restrict__ cu_dst, int nseq) {
   extern __shared__ uint4 sw[];
   pdl_trigger();
-  const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, stride = gridDim.x * kWarpsPerBlock;
   stage_norm_weights(w, vec, sw);
   pdl_wait();
   src = after_wait(src);
-  tok = after_wait(tok);
-  idx = after_wait(idx);
+  idx = after_wait(idx != nullptr ? idx : tok);
   pos_in = after_wait(pos_in);
-  if (r >= rows) return;
-  size_t srow;
-  int p;
-  if (idx == nullptr) {
-    int t = tok[r];
-    if (t < 0 || t >= vocab) {
-      if (lane == 0 && status != nullptr) atomicOr(status, kStatusBadIndex);
-      t = 0;
-    }
-    srow = static_cast<size_t>(t);
-    p = cu_dst ? r - __ldg(cu_dst + seq_of_row(cu_dst, nseq, r)) : r % L;
-  } else {
-    int b, n_b;
-    size_t row0;
-    if (cu_dst) {  // packed sequences of different lengths
-      b = seq_of_row(cu_dst, nseq, r);
+  int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+  int j = r < rows ? idx[r] : 0;
+  for (; r < rows; r += stride) {
+    const int next = r + stride < rows ? idx[r + stride] : 0;
+    const int b = cu_dst ? seq_of_row(cu_dst, nseq, r) : 0;  // packed sequences of different lengths
+    size_t row0 = 0;
+    int n = vocab;
+    if (tok == nullptr && cu_dst) {
       row0 = static_cast<size_t>(__ldg(cu_src + b));
-      n_b = __ldg(cu_src + b + 1) - __ldg(cu_src + b);
-    } else {
-      b = r / k;
-      row0 = static_cast<size_t>(b) * N;
-      n_b = N;
+      n = __ldg(cu_src + b + 1) - static_cast<int>(row0);
+    } else if (tok == nullptr) {
+      row0 = static_cast<size_t>(r / k) * N;
+      n = N;
     }
-    int j = idx[r];
-    if (j < 0 || j >= n_b) {
+    if (j < 0 || j >= n) {
       if (lane == 0 && status != nullptr) atomicOr(status, kStatusBadIndex);
       j = 0;
     }
-    srow = row0 + j;
-    p = pos_in[srow];
+    const uint4* sr = src + (row0 + j) * vec;
+    uint4 u[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (lane + 32 * q < vec) u[q] = sr[lane + 32 * q];
+    int p = 0;
+    if (lane == 0)
+      p = tok == nullptr ? pos_in[row0 + j] : cu_dst ? r - __ldg(cu_dst + b) : r % L;
+    uint4* hr = h_out + static_cast<size_t>(r) * vec;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (lane + 32 * q < vec) hr[lane + 32 * q] = u[q];
+    const float inv = row_inv_rms<Q>(u, lane, vec, eps);
+    write_normed<Q>(u, inv, sw, lane, vec, x_out + static_cast<size_t>(r) * vec);
+    if (lane == 0) pos_out[r] = p;
+    j = next;
   }
-  const uint4* sr = src + srow * vec;
-  uint4* hr = h_out + static_cast<size_t>(r) * vec;
-  uint4* xr = x_out + static_cast<size_t>(r) * vec;
-  uint4 u[kMaxVecPerLane];
-  float ss = 0.f;
-#pragma unroll
-  for (int q = 0; q < kMaxVecPerLane; ++q) {
-    const int v = lane + 32 * q;
-    if (v < vec) {
-      u[q] = sr[v];
-      hr[v] = u[q];
-      const uint32_t e4[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float a = bf16lo(e4[e]), c = bf16hi(e4[e]);
-        ss += a * a + c * c;
-      }
-    }
-  }
-  ss = warp_sum(ss);
-  const float inv = rsqrtf(ss / static_cast<float>(vec * 8) + eps);
-#pragma unroll
-  for (int q = 0; q < kMaxVecPerLane; ++q) {
-    const int v = lane + 32 * q;
-    if (v < vec) {
-      const uint4 wv = sw[v];
-      const uint32_t e4[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
-      const uint32_t w4[4] = {wv.x, wv.y, wv.z, wv.w};
-      uint32_t o[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        o[e] = pack_bf16x2(bf16lo(e4[e]) * inv * bf16lo(w4[e]), bf16hi(e4[e]) * inv * bf16hi(w4[e]));
-      xr[v] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-  }
-  if (lane == 0) pos_out[r] = p;
 }
 
 // ---------------------------------------------------------------- RoPE (fp32 path)
@@ -683,9 +696,13 @@ cudaError_t launch_embed(int dtype, const void* E, const int32_t* tok, int rows,
 cudaError_t launch_rmsnorm(int dtype, const void* h, const void* w, int rows, int d, float eps,
                            void* x, cudaStream_t s) {
   if (dtype == ZSAA_BF16 && d % 8 == 0 && d / 8 <= 32 * kMaxVecPerLane) {
-    ZSAA_LAUNCH(rmsnorm_bf16_reg_kernel, dim3(row_blocks(rows)), dim3(32 * kWarpsPerBlock),
-                static_cast<size_t>(d / 8) * 16, s, static_cast<const uint4*>(h), static_cast<const uint4*>(w),
-                rows, d / 8, eps, static_cast<uint4*>(x));
+    return norm_dispatch(d / 8, [&](auto q) -> cudaError_t {
+      constexpr int Q = decltype(q)::value;
+      ZSAA_LAUNCH(rmsnorm_bf16_reg_kernel<Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
+                  static_cast<size_t>(d / 8) * 16, s, static_cast<const uint4*>(h), static_cast<const uint4*>(w),
+                  rows, d / 8, eps, static_cast<uint4*>(x));
+      return cudaGetLastError();
+    });
   } else if (dtype == ZSAA_BF16 && d % 8 == 0) {
     ZSAA_LAUNCH(rmsnorm_bf16_vec_kernel, dim3(row_blocks(rows)), dim3(32 * kWarpsPerBlock), 0, s, 
         static_cast<const uint4*>(h), static_cast<const uint4*>(w), rows, d / 8, eps,
@@ -774,12 +791,14 @@ cudaError_t launch_rows_norm(const void* src, const int32_t* tok, int vocab, int
                              int d, const void* w, float eps, void* h_out, void* x_out,
                              int32_t* pos_out, int* status, cudaStream_t s, const int* cu_src,
                              const int* cu_dst, int nseq) {
-  ZSAA_LAUNCH(rows_norm_bf16_kernel, dim3(row_blocks(rows)), dim3(32 * kWarpsPerBlock),
-              static_cast<size_t>(d / 8) * 16, s,
-              static_cast<const uint4*>(src), tok, vocab, L, idx, N, k, pos_in, rows, d / 8,
-              static_cast<const uint4*>(w), eps, static_cast<uint4*>(h_out),
-              static_cast<uint4*>(x_out), pos_out, status, cu_src, cu_dst, nseq);
-  return cudaGetLastError();
+  return norm_dispatch(d / 8, [&](auto q) -> cudaError_t {
+    constexpr int Q = decltype(q)::value;
+    ZSAA_LAUNCH(rows_norm_bf16_kernel<Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
+                static_cast<size_t>(d / 8) * 16, s, static_cast<const uint4*>(src), idx == nullptr ? tok : nullptr,
+                vocab, L, idx, N, k, pos_in, rows, d / 8, static_cast<const uint4*>(w), eps,
+                static_cast<uint4*>(h_out), static_cast<uint4*>(x_out), pos_out, status, cu_src, cu_dst, nseq);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_gather(const void* src, int B, int N, int k, int row_bytes, const int32_t* idx,
