@@ -26,7 +26,9 @@ inline int row_blocks(int rows) { return (rows + kWarpsPerBlock - 1) / kWarpsPer
 // block staged the norm weights for eight rows only: embedding and norm of 16384
 // rows of 2048 took 61 us with events (3.3 TB/s), compaction and norm 20 us on
 // average over a forward; Q by the row length and a row loop 36 us (5.6 TB/s) and
-// 13 us.
+// 13 us.  Float rows (two passes of 4-byte loads, embedding and compaction as
+// kernels of their own): 11.6 us a norm of 324-1536 rows of 1024, here 6.7; and
+// two launches fewer in the 2-layer model, 78 -> 73 us a forward.
 __host__ __device__ constexpr int norm_blocks_per_sm(int Q) { return Q >= 16 ? 2 : Q >= 8 ? 4 : 6; }
 
 inline int norm_grid(int rows, int Q) {
@@ -42,21 +44,23 @@ inline int norm_grid(int rows, int Q) {
   return std::min(row_blocks(rows), sms * norm_blocks_per_sm(Q));
 }
 
-// fn(std::integral_constant<int, Q>) for the smallest Q that holds vec vectors: a
-// larger one costs registers (resident warps) and predicated-off instructions
-template <class Fn>
-cudaError_t norm_dispatch(int vec, Fn&& fn) {
-  if (vec <= 64) return fn(std::integral_constant<int, 2>());
-  if (vec <= 128) return fn(std::integral_constant<int, 4>());
-  if (vec <= 256) return fn(std::integral_constant<int, 8>());
-  return fn(std::integral_constant<int, kMaxVecPerLane>());
+// fn(a value of the element type, std::integral_constant<int, Q>) for the
+// smallest Q that holds a row of d: a larger one costs registers (resident
+// warps) and predicated-off instructions
+template <typename T, class Fn>
+cudaError_t norm_dispatch(T, int d, Fn&& fn) {
+  const int vec = d * static_cast<int>(sizeof(T)) / 16;
+  if (vec <= 64) return fn(T(), vec, std::integral_constant<int, 2>());
+  if (vec <= 128) return fn(T(), vec, std::integral_constant<int, 4>());
+  if (vec <= 256) return fn(T(), vec, std::integral_constant<int, 8>());
+  return fn(T(), vec, std::integral_constant<int, kMaxVecPerLane>());
 }
 
+template <class Fn>
+cudaError_t norm_dispatch(int dtype, int d, Fn&& fn) {
+  return dtype == ZSAA_BF16 ? norm_dispatch(bf16(), d, fn) : norm_dispatch(float(), d, fn);
+}
 
-// ---------------------------------------------------------------- embedding
-
-// h[r, :] = E[tok[r], :], pos[r] = r mod L  (a row is d * elem bytes, copied as uint4)
-// A token id outside [0, vocab) sets kStatusBadIndex and embeds row 0.
 __global__ void embed_kernel(const uint4* __restrict__ E, const int32_t* __restrict__ tok, int rows,
                              int L, int vocab, int vec_per_row, uint4* __restrict__ h,
                              int32_t* __restrict__ pos, int* status) {
@@ -117,52 +121,70 @@ __device__ __forceinline__ void stage_norm_weights(const uint4* __restrict__ w, 
   __syncthreads();
 }
 
+// The elements of a 16-byte vector: 8 bf16 or 4 float.
+template <typename T>
+constexpr int kVecElems = 16 / static_cast<int>(sizeof(T));
+
+template <typename T>
+__device__ __forceinline__ void unpack_vec(const uint4& u, float (&f)[kVecElems<T>]) {
+  const uint32_t e4[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if constexpr (kVecElems<T> == 8)
+      f[2 * e] = bf16lo(e4[e]), f[2 * e + 1] = bf16hi(e4[e]);
+    else
+      f[e] = __uint_as_float(e4[e]);
+  }
+}
+
 // 1/rms of a row held as Q vectors a lane (lane's vector q: lane + 32 q).
-template <int Q>
+template <typename T, int Q>
 __device__ __forceinline__ float row_inv_rms(const uint4 (&u)[Q], int lane, int vec, float eps) {
   float ss = 0.f;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     if (lane + 32 * q < vec) {
-      const uint32_t e4[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
+      float f[kVecElems<T>];
+      unpack_vec<T>(u[q], f);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float a = bf16lo(e4[e]), c = bf16hi(e4[e]);
-        ss += a * a + c * c;
-      }
+      for (int e = 0; e < kVecElems<T>; e += 2) ss += f[e] * f[e] + f[e + 1] * f[e + 1];
     }
   }
   ss = warp_sum(ss);
-  return rsqrtf(ss / static_cast<float>(vec * 8) + eps);
+  return rsqrtf(ss / static_cast<float>(vec * kVecElems<T>) + eps);
 }
 
 // x = h * inv * w of such a row, the weights in shared memory
-template <int Q>
+template <typename T, int Q>
 __device__ __forceinline__ void write_normed(const uint4 (&u)[Q], float inv, const uint4* sw, int lane, int vec,
                                              uint4* __restrict__ xr) {
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int v = lane + 32 * q;
     if (v < vec) {
-      const uint4 wv = sw[v];
-      const uint32_t e4[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
-      const uint32_t w4[4] = {wv.x, wv.y, wv.z, wv.w};
+      float f[kVecElems<T>], g[kVecElems<T>];
+      unpack_vec<T>(u[q], f);
+      unpack_vec<T>(sw[v], g);
       uint32_t o[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        o[e] = pack_bf16x2(bf16lo(e4[e]) * inv * bf16lo(w4[e]), bf16hi(e4[e]) * inv * bf16hi(w4[e]));
+      for (int e = 0; e < 4; ++e) {
+        if constexpr (kVecElems<T> == 8)
+          o[e] = pack_bf16x2(f[2 * e] * inv * g[2 * e], f[2 * e + 1] * inv * g[2 * e + 1]);
+        else
+          o[e] = __float_as_uint(f[e] * inv * g[e]);
+      }
       xr[v] = make_uint4(o[0], o[1], o[2], o[3]);
     }
   }
 }
 
-// bf16 rows of at most 32 Q vectors: one warp per row, the row loaded into
-// registers once (every load of a lane in flight together), its sum of
-// squares, then x = h / rms * w with the weights from shared memory.
-template <int Q>
+// Rows of at most 32 Q vectors: one warp per row, the row loaded into registers
+// once (every load of a lane in flight together), its sum of squares, then
+// x = h / rms * w with the weights from shared memory.
+template <typename T, int Q>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, norm_blocks_per_sm(Q))
-    rmsnorm_bf16_reg_kernel(const uint4* __restrict__ h, const uint4* __restrict__ w, int rows, int vec, float eps,
-                            uint4* __restrict__ x) {
+    rmsnorm_reg_kernel(const uint4* __restrict__ h, const uint4* __restrict__ w, int rows, int vec, float eps,
+                       uint4* __restrict__ x) {
   extern __shared__ uint4 sw[];
   pdl_trigger();
   stage_norm_weights(w, vec, sw);
@@ -175,8 +197,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, norm_blocks_per_sm(Q))
 #pragma unroll
     for (int q = 0; q < Q; ++q)
       if (lane + 32 * q < vec) u[q] = hr[lane + 32 * q];
-    const float inv = row_inv_rms<Q>(u, lane, vec, eps);
-    write_normed<Q>(u, inv, sw, lane, vec, x + static_cast<size_t>(r) * vec);
+    const float inv = row_inv_rms<T, Q>(u, lane, vec, eps);
+    write_normed<T, Q>(u, inv, sw, lane, vec, x + static_cast<size_t>(r) * vec);
   }
 }
 
@@ -557,19 +579,19 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ src, int N, int k, 
 // ---------------------------------------------------------------- row copy + RMSNorm
 
 // Copies source rows into the residual buffer and writes their RMSNorm, for
-// bf16 rows of d = 8 * vec elements (vec <= 32 * kMaxVecPerLane):
+// rows of vec 16-byte vectors (vec <= 32 * kMaxVecPerLane):
 //   embedding (idx == nullptr): source row tok[r] of E, pos_out[r] = r mod L;
 //   compaction: source row b*N + idx[r] of h (b = r / k), pos_out[r] =
 //     pos_in[that row] -- the kept rows of the previous layer, already normed
 //     for the next layer's attention.
 // An index outside its range sets kStatusBadIndex and copies row 0.
-template <int Q>
+template <typename T, int Q>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, norm_blocks_per_sm(Q))
-    rows_norm_bf16_kernel(const uint4* __restrict__ src, const int32_t* __restrict__ tok, int vocab, int L,
-                          const int32_t* __restrict__ idx, int N, int k, const int32_t* __restrict__ pos_in, int rows,
-                          int vec, const uint4* __restrict__ w, float eps, uint4* __restrict__ h_out,
-                          uint4* __restrict__ x_out, int32_t* __restrict__ pos_out, int* status,
-                          const int* __restrict__ cu_src, const int* __restrict__ cu_dst, int nseq) {
+    rows_norm_kernel(const uint4* __restrict__ src, const int32_t* __restrict__ tok, int vocab, int L,
+                     const int32_t* __restrict__ idx, int N, int k, const int32_t* __restrict__ pos_in, int rows,
+                     int vec, const uint4* __restrict__ w, float eps, uint4* __restrict__ h_out,
+                     uint4* __restrict__ x_out, int32_t* __restrict__ pos_out, int* status,
+                     const int* __restrict__ cu_src, const int* __restrict__ cu_dst, int nseq) {
   extern __shared__ uint4 sw[];
   pdl_trigger();
   const int lane = threadIdx.x & 31, stride = gridDim.x * kWarpsPerBlock;
@@ -608,8 +630,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, norm_blocks_per_sm(Q))
 #pragma unroll
     for (int q = 0; q < Q; ++q)
       if (lane + 32 * q < vec) hr[lane + 32 * q] = u[q];
-    const float inv = row_inv_rms<Q>(u, lane, vec, eps);
-    write_normed<Q>(u, inv, sw, lane, vec, x_out + static_cast<size_t>(r) * vec);
+    const float inv = row_inv_rms<T, Q>(u, lane, vec, eps);
+    write_normed<T, Q>(u, inv, sw, lane, vec, x_out + static_cast<size_t>(r) * vec);
     if (lane == 0) pos_out[r] = p;
     j = next;
   }
@@ -693,14 +715,20 @@ cudaError_t launch_embed(int dtype, const void* E, const int32_t* tok, int rows,
   return cudaGetLastError();
 }
 
+bool rows_norm_supported(int dtype, int d) {
+  const int bytes = d * (dtype == ZSAA_BF16 ? 2 : 4);
+  return bytes % 16 == 0 && bytes / 16 <= 32 * kMaxVecPerLane;
+}
+
 cudaError_t launch_rmsnorm(int dtype, const void* h, const void* w, int rows, int d, float eps,
                            void* x, cudaStream_t s) {
-  if (dtype == ZSAA_BF16 && d % 8 == 0 && d / 8 <= 32 * kMaxVecPerLane) {
-    return norm_dispatch(d / 8, [&](auto q) -> cudaError_t {
+  if (rows_norm_supported(dtype, d)) {
+    return norm_dispatch(dtype, d, [&](auto t, int vec, auto q) -> cudaError_t {
+      using T = decltype(t);
       constexpr int Q = decltype(q)::value;
-      ZSAA_LAUNCH(rmsnorm_bf16_reg_kernel<Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
-                  static_cast<size_t>(d / 8) * 16, s, static_cast<const uint4*>(h), static_cast<const uint4*>(w),
-                  rows, d / 8, eps, static_cast<uint4*>(x));
+      ZSAA_LAUNCH(rmsnorm_reg_kernel<T, Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
+                  static_cast<size_t>(vec) * 16, s, static_cast<const uint4*>(h), static_cast<const uint4*>(w), rows,
+                  vec, eps, static_cast<uint4*>(x));
       return cudaGetLastError();
     });
   } else if (dtype == ZSAA_BF16 && d % 8 == 0) {
@@ -786,16 +814,17 @@ cudaError_t launch_flags_from_idx(const int32_t* idx, int B, int N, int k, uint8
   return cudaGetLastError();
 }
 
-cudaError_t launch_rows_norm(const void* src, const int32_t* tok, int vocab, int L,
+cudaError_t launch_rows_norm(int dtype, const void* src, const int32_t* tok, int vocab, int L,
                              const int32_t* idx, int N, int k, const int32_t* pos_in, int rows,
                              int d, const void* w, float eps, void* h_out, void* x_out,
                              int32_t* pos_out, int* status, cudaStream_t s, const int* cu_src,
                              const int* cu_dst, int nseq) {
-  return norm_dispatch(d / 8, [&](auto q) -> cudaError_t {
+  return norm_dispatch(dtype, d, [&](auto t, int vec, auto q) -> cudaError_t {
+    using T = decltype(t);
     constexpr int Q = decltype(q)::value;
-    ZSAA_LAUNCH(rows_norm_bf16_kernel<Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
-                static_cast<size_t>(d / 8) * 16, s, static_cast<const uint4*>(src), idx == nullptr ? tok : nullptr,
-                vocab, L, idx, N, k, pos_in, rows, d / 8, static_cast<const uint4*>(w), eps,
+    ZSAA_LAUNCH(rows_norm_kernel<T, Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
+                static_cast<size_t>(vec) * 16, s, static_cast<const uint4*>(src), idx == nullptr ? tok : nullptr,
+                vocab, L, idx, N, k, pos_in, rows, vec, static_cast<const uint4*>(w), eps,
                 static_cast<uint4*>(h_out), static_cast<uint4*>(x_out), pos_out, status, cu_src, cu_dst, nseq);
     return cudaGetLastError();
   });

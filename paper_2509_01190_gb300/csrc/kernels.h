@@ -30,15 +30,17 @@ cudaError_t launch_select_parts(const float* parts, int n_qc, int B, int G, int 
 // alive (masked mode, fixed length): [B, N] flags; only flagged rows compete
 // (k includes the forced last row), and afterwards exactly the kept rows are
 // flagged.  idx then holds positions 0..N-1.
-// bf16 rows: h_out[r] = source row, x_out[r] = RMSNorm(h_out[r]) * w, pos_out[r].
+// h_out[r] = source row, x_out[r] = RMSNorm(h_out[r]) * w, pos_out[r].
 // Embedding when idx == nullptr (rows = B*L, source row tok[r] of E);
 // otherwise compaction (rows = B*k, source row b*N + idx[r] of h).
-// d % 8 == 0 and d <= kRowsNormMaxD.
+// Rows of whole 16-byte vectors, at most 512 of them (bf16: d % 8 == 0 and
+// d <= kRowsNormMaxD; float: d % 4 == 0 and half of that).
 constexpr int kRowsNormMaxD = 8 * 32 * 16;
+bool rows_norm_supported(int dtype, int d);
 // Variable length: cu_dst (offsets of the written rows; nseq sequences) gives
 // the sequence of a row and, for the embedding, pos = r - cu_dst[b]; cu_src
 // (offsets of the source rows) places compaction index j at row cu_src[b] + j.
-cudaError_t launch_rows_norm(const void* src, const int32_t* tok, int vocab, int L,
+cudaError_t launch_rows_norm(int dtype, const void* src, const int32_t* tok, int vocab, int L,
                              const int32_t* idx, int N, int k, const int32_t* pos_in, int rows,
                              int d, const void* w, float eps, void* h_out, void* x_out,
                              int32_t* pos_out, int* status, cudaStream_t s,

@@ -555,14 +555,14 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
       ZCK(cudaStreamSynchronize(s));
     }
   }
-  // bf16 rows of moderate width: embedding and compaction also write the next
+  // Rows of moderate width: embedding and compaction also write the next
   // layer's normed input (x_ready), saving that layer's RMSNorm launch.
-  const bool fuse_norm = dt == ZSAA_BF16 && d % 8 == 0 && d <= kRowsNormMaxD;
+  const bool fuse_norm = rows_norm_supported(dt, static_cast<int>(d));
   bool x_ready = false;
   if (!from_hidden) {
     if (fuse_norm && first <= n_run) {
       TRACE("embed_norm", 0.0, static_cast<double>(B) * L * (3.0 * d * es + 8.0));
-      ZCK(launch_rows_norm(m->embed, tok, c.vocab, L, nullptr, 0, 0, nullptr, B * L, d,
+      ZCK(launch_rows_norm(dt, m->embed, tok, c.vocab, L, nullptr, 0, 0, nullptr, B * L, d,
                            LW(m, first - 1, kAttnNorm), c.rms_eps, m->h[cur], m->x, m->pos[cur],
                            m->status, s));
       x_ready = true;
@@ -708,7 +708,7 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
           if (fork) ZCK(cudaStreamWaitEvent(s, m->ev_join, 0));  // the O-projection has updated h
           if (fuse_norm) {  // the kept rows and their pre-MLP RMSNorm in one pass
             TRACE("gather_norm", 0.0, static_cast<double>(B) * k * (3.0 * d * es + 12.0));
-            ZCK(launch_rows_norm(h, nullptr, 0, 0, idx, N, k, m->pos[cur], B * k, d,
+            ZCK(launch_rows_norm(dt, h, nullptr, 0, 0, idx, N, k, m->pos[cur], B * k, d,
                                  LW(m, li, kMlpNorm), c.rms_eps, m->h[cur ^ 1], m->x,
                                  m->pos[cur ^ 1], m->status, s));
             mlp_x_ready = true;
@@ -771,7 +771,7 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
   if (kc != nullptr) {  // next-token logits: final norm and LM head of the last kept row
     if (fuse_norm) {
       TRACE("gather_norm", 0.0, static_cast<double>(B) * (3.0 * d * es + 12.0));
-      ZCK(launch_rows_norm(m->h[cur], nullptr, 0, 0, kc->last_idx, N, 1, m->pos[cur], B, d,
+      ZCK(launch_rows_norm(dt, m->h[cur], nullptr, 0, 0, kc->last_idx, N, 1, m->pos[cur], B, d,
                            m->final_norm, c.rms_eps, m->h[cur ^ 1], m->x, m->pos[cur ^ 1],
                            m->status, s));
     } else {
@@ -881,7 +881,7 @@ zsaa_status run_forward_masked(zsaa_model* m, const int32_t* tok, int B, int L, 
 #define TRACE(name, fl, by) TraceScope trace_scope_(m, name, fl, by, s)
   {
     TRACE("embed_norm", 0.0, Md * (3.0 * d * es + 8.0));
-    ZCK(launch_rows_norm(m->embed, tok, c.vocab, L, nullptr, 0, 0, nullptr, M, d,
+    ZCK(launch_rows_norm(dt, m->embed, tok, c.vocab, L, nullptr, 0, 0, nullptr, M, d,
                          LW(m, 0, kAttnNorm), c.rms_eps, h, m->x, m->pos[0], m->status, s));
   }
   const int32_t* kept = nullptr;  // positions of the unmarked rows after the last selection
@@ -1020,7 +1020,7 @@ zsaa_status run_forward_masked(zsaa_model* m, const int32_t* tok, int B, int L, 
   const int32_t* posf = m->pos[0];
   if (kept != nullptr) {
     TRACE("gather_norm", 0.0, static_cast<double>(B) * nf * (3.0 * d * es + 12.0));
-    ZCK(launch_rows_norm(h, nullptr, 0, 0, kept, L, nf, m->pos[0], B * nf, d, m->final_norm,
+    ZCK(launch_rows_norm(dt, h, nullptr, 0, 0, kept, L, nf, m->pos[0], B * nf, d, m->final_norm,
                          c.rms_eps, m->h[1], m->x, m->pos[1], m->status, s));
     hf = m->h[1];
     posf = m->pos[1];
@@ -1111,7 +1111,7 @@ zsaa_status run_forward_varlen(zsaa_model* m, const int32_t* tok, const int32_t*
 #define TRACE(name, fl, by) TraceScope trace_scope_(m, name, fl, by, s)
   {
     TRACE("embed_norm", 0.0, static_cast<double>(T0) * (3.0 * d * es + 8.0));
-    ZCK(launch_rows_norm(m->embed, tok, c.vocab, 1, nullptr, 0, 0, nullptr, rows[0], d,
+    ZCK(launch_rows_norm(dt, m->embed, tok, c.vocab, 1, nullptr, 0, 0, nullptr, rows[0], d,
                          LW(m, 0, kAttnNorm), c.rms_eps, m->h[cur], m->x, m->pos[cur], m->status,
                          s, nullptr, cu_dev(0), B));
   }
@@ -1205,7 +1205,7 @@ zsaa_status run_forward_varlen(zsaa_model* m, const int32_t* tok, const int32_t*
         if (shrinks) {
           if (fork) ZCK(cudaStreamWaitEvent(s, m->ev_join, 0));  // the O-projection has updated h
           TRACE("gather_norm", 0.0, static_cast<double>(rows[l]) * (3.0 * d * es + 12.0));
-          ZCK(launch_rows_norm(h, nullptr, 0, 0, idx, Nm, 0, m->pos[cur], rows[l], d,
+          ZCK(launch_rows_norm(dt, h, nullptr, 0, 0, idx, Nm, 0, m->pos[cur], rows[l], d,
                                LW(m, li, kMlpNorm), c.rms_eps, m->h[cur ^ 1], m->x, m->pos[cur ^ 1],
                                m->status, s, cu_dev(li), cu_dev(l), B));
           mlp_x_ready = true;
@@ -1462,7 +1462,7 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
 #define TRACE(name, fl, by) TraceScope trace_scope_(m, name, fl, by, s)
   {
     TRACE("embed_norm", 0.0, Bd * (3.0 * d * es + 8.0));
-    ZCK(launch_rows_norm(m->embed, tok, c.vocab, 1, nullptr, 0, 0, nullptr, B, d,
+    ZCK(launch_rows_norm(c.dtype, m->embed, tok, c.vocab, 1, nullptr, 0, 0, nullptr, B, d,
                          LW(m, 0, kAttnNorm), c.rms_eps, h, m->x, m->pos[0], m->status, s));
   }
   for (int li = 0; li < c.n_layers; ++li) {

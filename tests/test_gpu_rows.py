@@ -4,6 +4,8 @@ lane holds (2, 4, 8, 16 vectors), more rows than the resident warps, and packed
 batches of more sequences than one (32) and two (1024) rounds of the search for
 a row's sequence."""
 
+import dataclasses
+
 import pytest
 
 from paper_2509_01190_gb300 import inputs as I
@@ -42,3 +44,13 @@ def test_rows_and_norms(z, d, B, L):
 def test_packed_rows_of_many_sequences(z, B):
     lengths = [1 + (7 * b) % 5 for b in range(B)]
     check_varlen(run_varlen_case(z, SMALL_BF16, lengths, 1.5), SMALL_BF16)
+
+
+# float rows: 4 elements a vector, so the same lengths at half the width; past
+# d 2048 the embedding, the compaction and the norm are kernels of their own.
+@pytest.mark.parametrize("d,B,L", [(256, 3, 67), (272, 2, 33), (256, 200, 79), (1024, 161, 63), (1040, 81, 63),
+                                   (2048, 2, 33), (2064, 2, 33)])
+def test_rows_and_norms_f32(z, d, B, L):
+    shape = dataclasses.replace(I.TINY_F32, name="rows-f32-%d" % d, d_model=d, n_heads=4, n_kv_heads=2, head_dim=32,
+                                ffn_dim=200, vocab=333)
+    check_case(run_case(z, shape, B, L, 2.0, seqs=[0, B - 1]), "f32")
