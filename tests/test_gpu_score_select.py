@@ -63,6 +63,33 @@ def test_selector_fed_scores_matches_oracle_exactly(z, B, L):
                 np.testing.assert_array_equal(idx.cpu().numpy(), ref, err_msg=f"k={k} fl={fl}")
 
 
+# Both sides of each block size and of the register route's 4 candidates a
+# thread, with keys whose highest differing bit is anywhere: all equal, one
+# apart from the rest, neighbours in the last bits, every exponent, both signs.
+@pytest.mark.parametrize("L", [258, 259, 511, 512, 513, 1025, 1537, 2047, 2048, 2049, 4096, 4097, 4098, 5000])
+def test_selector_key_ranges_match_oracle_exactly(z, L):
+    rng = np.random.default_rng(L)
+    one = np.float32(1.0)
+    rows = [np.full(L, 0.25, np.float32),
+            np.where(np.arange(L) == L // 2, np.float32(-3.0), one).astype(np.float32),
+            (one + rng.integers(0, 300, L).astype(np.float32) * np.float32(2.0 ** -23)).astype(np.float32),
+            np.ldexp(rng.random(L) + 1.0, rng.integers(-120, 120, L)).astype(np.float32) *
+            rng.choice([-1.0, 1.0], L).astype(np.float32),
+            (34.0 + 0.7 * rng.standard_normal(L)).astype(np.float32),
+            np.where(rng.random(L) < 0.5, np.float32(np.nan), rng.integers(0, 2, L)).astype(np.float32)]
+    sc = np.stack(rows)
+    B = len(rows)
+    hidden = torch.zeros(B, L, 8, device="cuda", dtype=torch.bfloat16)
+    s_dev = torch.from_numpy(sc).cuda()
+    for k in (1, 2, 7, L // 11, L // 4, L // 2, L - 2, L - 1, L):
+        for fl in (0, 1):
+            idx = torch.empty(B, k, device="cuda", dtype=torch.int32)
+            z.zsaa_score_select_ex(hidden, B, L, 8, z.ZSAA_BF16, k, fl, s_dev, None, idx)
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(idx.cpu().numpy(), _select_oracle_f32(sc, k, bool(fl)),
+                                          err_msg=f"k={k} fl={fl}")
+
+
 def _check_scores_and_idx(hidden_np, scores_gpu, idx_gpu, k, force_last, bs):
     for b in bs:
         s_ref = np.sqrt(np.sum(hidden_np[b].astype(np.float64) ** 2, axis=-1))
