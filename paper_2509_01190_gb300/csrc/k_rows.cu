@@ -309,7 +309,7 @@ __device__ __forceinline__ uint32_t order_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-constexpr int kKeysPerThread = 4;
+constexpr int kRankMax = 112;
 
 // One block per sequence, of THREADS threads (256 to 1024, by the sequence
 // length: the selection is a chain of block-wide barriers, which cost less in
@@ -317,25 +317,27 @@ constexpr int kKeysPerThread = 4;
 // the few hundred kept rows of the deep pruned layers).  Radix select (passes of 8 bits) finds the key T of
 // the need-th best candidate and how many candidates equal to T are taken;
 // then an index-ordered prefix scan writes the kept indices ascending.
-//  - Up to 256 candidates without marks: each thread counts its candidate's rank
-//    against all others.
-//  - Up to 4 per thread (kKeysPerThread): a thread keeps four neighbouring keys
-//    in registers.  The passes start at the highest bit in which the smallest
-//    and the largest key differ (scores share sign and exponent: their first 8
-//    bits would put nearly all of them into one bin, an atomic at a time) and
-//    end when a bin is taken whole, which two passes nearly always reach; two
+//  - Up to kRankMax candidates without marks: each thread counts its candidate's
+//    rank against all others (100: 2.4 us back to back against 2.6; 128: 2.7
+//    against 2.5; 256: 4.2 against 2.4).
+//  - Up to KPT candidates a thread: a thread keeps KPT neighbouring keys in
+//    registers.  The passes start at the highest bit in which the smallest and
+//    the largest key differ (scores share sign and exponent: their first 8 bits
+//    would put nearly all of them into one bin, an atomic at a time) and end
+//    when a bin is taken whole, which two passes nearly always reach; two
 //    barriers a pass and one block-wide scan.  What bounds it is this chain of
-//    barriers.
-//    Isolated on 3 x 1537 float rows (norms, selection, rows): 13.5 -> 11.2 us
-//    against the form below; 4 x 2048 in a forward: 14.8 -> 12.4 us with events.
-//  - Longer (registers would not hold the keys): four passes from the top bit,
-//    keys re-read in each, and a scan per THREADS candidates.
+//    barriers.  8 sequences of 400 / 2048 / 4096 scores back to back: 4.6 / 6.5 /
+//    7.9 us with four passes from the top bit and a scan per THREADS candidates,
+//    here 2.7 / 3.1 / 4.4; 3 x 1537 float rows with
+//    their norms and compaction 13.5 -> 11.2.
+//  - KPT = 0, longer sequences (the registers would not hold the keys): the same,
+//    in chunks of four keys a thread that are read again in each pass.
 // Ties (equal keys) keep lower indices first.  With force_last the last index
 // is kept and the other k-1 come from indices [0, N-1).
 // FROM_PARTS: the scores are first summed from column-mass partials
 // parts[qc][b][g][j] (n_qc chunks, G groups) into shared memory (and copied to
 // scores_out when it is not null); otherwise they are read from `scores`.
-template <bool FROM_PARTS, int THREADS>
+template <bool FROM_PARTS, int THREADS, int KPT>
 __global__ void __launch_bounds__(THREADS)
     select_topk_kernel(const float* __restrict__ scores, int Ns, int ks, int force_last,
                        int32_t* __restrict__ idx_out, const float* __restrict__ parts, int n_qc,
@@ -405,11 +407,11 @@ __global__ void __launch_bounds__(THREADS)
 
   __shared__ __align__(16) uint32_t hist[512];
   __shared__ uint32_t sh_digit, sh_remaining, sh_count;
-  __shared__ int wgt[nwarps], weq[nwarps], wcount[nwarps];
-  __shared__ int tile_gt, tile_eq;
+  __shared__ int wgt[nwarps];
+  __shared__ uint32_t wlo[nwarps], whi[nwarps], wcount[2][nwarps];
   const uint32_t lt_mask = (1u << lane) - 1u;
 
-  if (THREADS == 256 && al == nullptr && n_cand <= THREADS) {
+  if (THREADS == 256 && al == nullptr && n_cand <= kRankMax) {
     // Short sequence, one candidate per thread: count the candidates ahead of
     // candidate j in (key descending, index ascending) order directly.  Rank <
     // need is the radix path's kept set (every key above the threshold, then
@@ -439,8 +441,6 @@ __global__ void __launch_bounds__(THREADS)
     return;
   }
 
-  // warp 0: the bin of h that holds the remaining-th largest, its count, and
-  // how many of it are still to be taken
   auto find_digit = [&](const uint32_t* h, uint32_t remaining) {
     uint32_t c[8], local = 0;
 #pragma unroll
@@ -465,53 +465,68 @@ __global__ void __launch_bounds__(THREADS)
       acc += c[q];
     }
   };
-  uint32_t prefix = 0, mask = 0, remaining = static_cast<uint32_t>(need);
-  if (n_cand <= kKeysPerThread * THREADS) {
-    const int j0 = tid * kKeysPerThread;
-    uint32_t key[kKeysPerThread];
-    bool in[kKeysPerThread];
-    uint32_t lo = 0xffffffffu, hi = 0u;
+  // the candidates' keys in chunks of KREG neighbouring ones a thread: a single
+  // chunk, or read again each time
+  constexpr int KREG = KPT > 0 ? KPT : 4;
+  uint32_t key[KREG];
+  bool in[KREG];
+  auto load_keys = [&](int j0) {
 #pragma unroll
-    for (int q = 0; q < kKeysPerThread; ++q) {
+    for (int q = 0; q < KREG; ++q) {
       in[q] = j0 + q < n_cand && (al == nullptr || al[j0 + q] != 0);
       key[q] = in[q] ? order_key(s[j0 + q]) : 0u;
-      if (in[q]) lo = min(lo, key[q]), hi = max(hi, key[q]);
     }
-    if (need > 0) {
-      lo = __reduce_min_sync(0xffffffffu, lo);
-      hi = __reduce_max_sync(0xffffffffu, hi);
-      if (lane == 0) wgt[warp] = static_cast<int>(lo), weq[warp] = static_cast<int>(hi);
-      for (int i = tid; i < 512; i += THREADS) hist[i] = 0;
+  };
+  if (KPT > 0) load_keys(tid * KREG);
+  auto each_key = [&](auto&& fn) {
+    for (int c0 = 0; c0 < (KPT > 0 ? 1 : n_cand); c0 += KREG * THREADS) {
+      if (KPT == 0) load_keys(c0 + tid * KREG);
+#pragma unroll
+      for (int q = 0; q < KREG; ++q)
+        if (in[q]) fn(key[q]);
+    }
+  };
+  if (need > 0) {
+    uint32_t lo = 0xffffffffu, hi = 0u, remaining = static_cast<uint32_t>(need);
+    each_key([&](uint32_t kj) { lo = min(lo, kj), hi = max(hi, kj); });
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) wlo[warp] = lo, whi[warp] = hi;
+    for (int i = tid; i < 512; i += THREADS) hist[i] = 0;
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lane < nwarps ? wlo[lane] : 0xffffffffu);
+    hi = __reduce_max_sync(0xffffffffu, lane < nwarps ? whi[lane] : 0u);
+    int top = 32 - __clz(lo ^ hi);  // the bits below top are undecided
+    uint32_t mask = top == 32 ? 0u : 0xffffffffu << top, prefix = hi & mask;
+    uint32_t* h = hist;
+    while (top > 0) {
+      const int low = max(top - 8, 0);
+      const uint32_t bins = (1u << (top - low)) - 1u;
+      each_key([&](uint32_t kj) {
+        if ((kj & mask) == prefix) atomicAdd(h + ((kj >> low) & bins), 1u);
+      });
       __syncthreads();
-      lo = __reduce_min_sync(0xffffffffu, lane < nwarps ? static_cast<uint32_t>(wgt[lane]) : 0xffffffffu);
-      hi = __reduce_max_sync(0xffffffffu, lane < nwarps ? static_cast<uint32_t>(weq[lane]) : 0u);
-      int top = 32 - __clz(lo ^ hi);  // the bits below top are undecided
-      mask = top == 32 ? 0u : 0xffffffffu << top;
-      prefix = hi & mask;
-      uint32_t* h = hist;
-      while (top > 0) {
-        const int low = max(top - 8, 0);
-        const uint32_t bins = (1u << (top - low)) - 1u;
+      uint32_t* next = hist + 256 - (h - hist);
+      if (warp == 0)  // the bin that holds the remaining-th largest, its count, how many of it to take
+        find_digit(h, remaining);
+      else
+        for (int i = tid - 32; i < 256; i += THREADS - 32) next[i] = 0;
+      __syncthreads();
+      prefix |= sh_digit << low;
+      mask = 0xffffffffu << low;
+      remaining = sh_remaining;
+      top = low;
+      h = next;
+      if (sh_count == remaining) break;  // the bin is taken whole
+    }
+    uint32_t base_gt = 0, base_eq = 0;
+    int buf = 0;
+    for (int c0 = 0; c0 < (KPT > 0 ? 1 : n_cand); c0 += KREG * THREADS, buf ^= 1) {
+      const int j0 = c0 + tid * KREG;
+      if (KPT == 0) load_keys(j0);
+      uint32_t n = 0;  // above the threshold << 16 | equal to it, then those before this thread's
 #pragma unroll
-        for (int q = 0; q < kKeysPerThread; ++q)
-          if (in[q] && (key[q] & mask) == prefix) atomicAdd(h + ((key[q] >> low) & bins), 1u);
-        __syncthreads();
-        uint32_t* next = hist + 256 - (h - hist);
-        if (warp == 0)
-          find_digit(h, remaining);
-        else
-          for (int i = tid - 32; i < 256; i += THREADS - 32) next[i] = 0;
-        __syncthreads();
-        prefix |= sh_digit << low;
-        mask = 0xffffffffu << low;
-        remaining = sh_remaining;
-        top = low;
-        h = next;
-        if (sh_count == remaining) break;  // the bin is taken whole
-      }
-      uint32_t n = 0;  // above T << 16 | equal to it, then those before this thread's
-#pragma unroll
-      for (int q = 0; q < kKeysPerThread; ++q)
+      for (int q = 0; q < KREG; ++q)
         if (in[q]) n += (key[q] & mask) > prefix ? 0x10000u : ((key[q] & mask) == prefix ? 1u : 0u);
       uint32_t before = n;
 #pragma unroll
@@ -519,12 +534,13 @@ __global__ void __launch_bounds__(THREADS)
         const uint32_t v = __shfl_up_sync(0xffffffffu, before, o);
         if (lane >= o) before += v;
       }
-      if (lane == 31) wcount[warp] = static_cast<int>(before);
+      if (lane == 31) wcount[buf][warp] = before;
       __syncthreads();
-      before += __reduce_add_sync(0xffffffffu, lane < warp ? static_cast<uint32_t>(wcount[lane]) : 0u) - n;
-      uint32_t gt = before >> 16, eq = before & 0xffffu;
+      const uint32_t w = lane < nwarps ? wcount[buf][lane] : 0u;
+      before += __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) - n;
+      uint32_t gt = base_gt + (before >> 16), eq = base_eq + (before & 0xffffu);
 #pragma unroll
-      for (int q = 0; q < kKeysPerThread; ++q) {
+      for (int q = 0; q < KREG; ++q) {
         const uint32_t mk = key[q] & mask;
         if (!in[q] || mk < prefix) continue;
         if (mk > prefix || eq < remaining) out[gt + min(eq, remaining)] = j0 + q;
@@ -533,69 +549,11 @@ __global__ void __launch_bounds__(THREADS)
         else
           ++eq;
       }
-    }
-  } else {
-    if (need > 0) {
-      for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 24 - 8 * pass;
-        for (int i = tid; i < 256; i += THREADS) hist[i] = 0;
-        __syncthreads();
-        for (int j = tid; j < n_cand; j += THREADS) {
-          if (al != nullptr && al[j] == 0) continue;  // masked mode: only unmarked rows compete
-          const uint32_t key = order_key(s[j]);
-          if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-        }
-        __syncthreads();
-        if (warp == 0) find_digit(hist, remaining);
-        __syncthreads();
-        prefix |= sh_digit << shift;
-        mask |= 255u << shift;
-        remaining = sh_remaining;
-        __syncthreads();
+      if (KPT == 0) {
+        const uint32_t all = __reduce_add_sync(0xffffffffu, w);
+        base_gt += all >> 16;
+        base_eq += all & 0xffffu;
       }
-    }
-    const uint32_t T = prefix;
-    int base_gt = 0, base_eq = 0;
-    for (int j0 = 0; j0 < n_cand && need > 0; j0 += THREADS) {
-      const int j = j0 + tid;
-      const bool in = j < n_cand && (al == nullptr || al[j] != 0);
-      const uint32_t key = in ? order_key(s[j]) : 0u;
-      const bool gt = in && key > T;
-      const bool eq = in && key == T;
-      const uint32_t bgt = __ballot_sync(0xffffffffu, gt), beq = __ballot_sync(0xffffffffu, eq);
-      if (lane == 0) {
-        wgt[warp] = __popc(bgt);
-        weq[warp] = __popc(beq);
-      }
-      __syncthreads();
-      if (warp == 0) {  // exclusive scan of the per-warp counts
-        int a = lane < nwarps ? wgt[lane] : 0, e = lane < nwarps ? weq[lane] : 0;
-        int ia = a, ie = e;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          int va = __shfl_up_sync(0xffffffffu, ia, o), ve = __shfl_up_sync(0xffffffffu, ie, o);
-          if (lane >= o) {
-            ia += va;
-            ie += ve;
-          }
-        }
-        if (lane < nwarps) {
-          wgt[lane] = ia - a;
-          weq[lane] = ie - e;
-        }
-        if (lane == 31) {
-          tile_gt = ia;
-          tile_eq = ie;
-        }
-      }
-      __syncthreads();
-      const int gt_before = base_gt + wgt[warp] + __popc(bgt & lt_mask);
-      const int eq_before = base_eq + weq[warp] + __popc(beq & lt_mask);
-      const int rem = static_cast<int>(remaining);
-      if (gt || (eq && eq_before < rem)) out[gt_before + min(eq_before, rem)] = j;
-      base_gt += tile_gt;
-      base_eq += tile_eq;
-      __syncthreads();
     }
   }
   if (force_last && tid == 0) out[k - 1] = N - 1;
@@ -846,39 +804,36 @@ cudaError_t launch_row_norm(int dtype, const void* h, int rows, int d, float* sc
   return cudaGetLastError();
 }
 
-// Threads of a selection block for sequences of up to N rows.
-inline int sel_threads(int N) { return N <= 512 ? 256 : (N <= 2048 ? 512 : 1024); }
-
-template <bool FROM_PARTS, int T>
+template <bool FROM_PARTS, int T, int KPT>
 cudaError_t launch_select_t(const float* scores, const float* parts, int n_qc, int B, int G, int N, int k,
                             int force_last, int32_t* idx, float* scores_out, size_t smem, cudaStream_t s,
                             const int* cu_in, const int* cu_out, uint8_t* alive) {
   if (FROM_PARTS) {
     static OncePerDevice once;
-    const cudaError_t attr = set_smem_limit_once(once, select_topk_kernel<true, T>,
+    const cudaError_t attr = set_smem_limit_once(once, select_topk_kernel<true, T, KPT>,
                                                  static_cast<int>(kSelectPartsMaxN * sizeof(float)));
     if (attr != cudaSuccess) return attr;
   }
-  ZSAA_LAUNCH(select_topk_kernel<FROM_PARTS, T>, dim3(B), dim3(T), smem, s, scores, N, k, force_last, idx, parts,
+  ZSAA_LAUNCH(select_topk_kernel<FROM_PARTS, T, KPT>, dim3(B), dim3(T), smem, s, scores, N, k, force_last, idx, parts,
               n_qc, B, G, scores_out, cu_in, cu_out, alive);
   return cudaGetLastError();
 }
 
+// N: rows of the longest sequence
 template <bool FROM_PARTS>
 cudaError_t launch_select_any(const float* scores, const float* parts, int n_qc, int B, int G, int N, int k,
                               int force_last, int32_t* idx, float* scores_out, size_t smem, cudaStream_t s,
                               const int* cu_in, const int* cu_out, uint8_t* alive) {
-  switch (sel_threads(N)) {
-    case 256:
-      return launch_select_t<FROM_PARTS, 256>(scores, parts, n_qc, B, G, N, k, force_last, idx, scores_out, smem,
-                                              s, cu_in, cu_out, alive);
-    case 512:
-      return launch_select_t<FROM_PARTS, 512>(scores, parts, n_qc, B, G, N, k, force_last, idx, scores_out, smem,
-                                              s, cu_in, cu_out, alive);
-    default:
-      return launch_select_t<FROM_PARTS, 1024>(scores, parts, n_qc, B, G, N, k, force_last, idx, scores_out,
-                                               smem, s, cu_in, cu_out, alive);
-  }
+  static_assert(kSelectPartsMaxN <= 12 * 1024, "the longest form that sums partials");
+  auto go = [&](auto launch) {
+    return launch(scores, parts, n_qc, B, G, N, k, force_last, idx, scores_out, smem, s, cu_in, cu_out, alive);
+  };
+  if (N <= 512) return go(launch_select_t<FROM_PARTS, 256, 4>);
+  if (N <= 2048) return go(launch_select_t<FROM_PARTS, 512, 4>);
+  if (N <= 4096) return go(launch_select_t<FROM_PARTS, 1024, 4>);
+  if (N <= 12 * 1024) return go(launch_select_t<FROM_PARTS, 1024, 12>);
+  if constexpr (!FROM_PARTS) return go(launch_select_t<false, 1024, 0>);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_select(const float* scores, int B, int N, int k, int force_last, int32_t* idx,

@@ -36,7 +36,7 @@ def _select_oracle_f32(scores32, k, force_last):
     return np.stack([O.select_topk(s[b], k, force_last) for b in range(s.shape[0])])
 
 
-# up to 256 candidates (L <= 256, or 257 with force-keep-last) take the rank-count
+# up to 112 candidates (L <= 112, or 113 with force-keep-last) take the rank-count
 # route, longer sequences the radix passes
 @pytest.mark.parametrize("B,L", [(3, 1), (2, 7), (2, 64), (3, 200), (2, 255), (2, 256), (2, 257), (4, 1000),
                                  (2, 1024), (1, 3001), (2, 8192)])
@@ -63,10 +63,11 @@ def test_selector_fed_scores_matches_oracle_exactly(z, B, L):
                 np.testing.assert_array_equal(idx.cpu().numpy(), ref, err_msg=f"k={k} fl={fl}")
 
 
-# Both sides of each block size and of the register route's 4 candidates a
-# thread, with keys whose highest differing bit is anywhere: all equal, one
+# Both sides of the rank count's limit, of each block size and of the register
+# route's 4 and 12 candidates a thread, with keys whose highest differing bit is anywhere: all equal, one
 # apart from the rest, neighbours in the last bits, every exponent, both signs.
-@pytest.mark.parametrize("L", [258, 259, 511, 512, 513, 1025, 1537, 2047, 2048, 2049, 4096, 4097, 4098, 5000])
+@pytest.mark.parametrize("L", [111, 112, 113, 114, 257, 511, 512, 513, 1025, 1537, 2047, 2048, 2049, 4096, 4097, 4098, 5000,
+                               12287, 12288, 12289, 15000])
 def test_selector_key_ranges_match_oracle_exactly(z, L):
     rng = np.random.default_rng(L)
     one = np.float32(1.0)
