@@ -57,12 +57,12 @@ TRAFFIC = {
     # profiles/gemm_gate_up_swiglu_8b_traffic.md: the first layer's MLP at accel 4
     ("gemm_gate_up_swiglu", "8b"): {
         "launch": "gate/up + SwiGLU, M=7272 rows (layer 1 of the accel-4 forward), N=2x14336, K=4096",
-        "bytes": 1343622912.0,
+        "bytes": 1383143936.0,
         "algorithmic_bytes": 502956032.0,
         "sources": {
-            "paper_2509_01190_gb300/csrc/k_gemm_tc.cu": "476652139b6316266382a408d78f0d679ecabad54bb26d64f2f15e01a1c5d7f0",
-            "paper_2509_01190_gb300/csrc/common.cuh": "9e474368fc0200765d2891a8fa691189a035962da12ffe00a8ef80d040644cbf",
-            "paper_2509_01190_gb300/csrc/kernels.h": "c895255d48b1cd8b7810c67d6c8082cc110807e30ffdb7a90ddc0a9faca5635b",
+            "paper_2509_01190_gb300/csrc/k_gemm_tc.cu": "3375275a6ffc203ecf76f450cd933fa48f17c5e8deb0f98d9d8d388b2570fb83",
+            "paper_2509_01190_gb300/csrc/common.cuh": "e629752c9039f4ede210522a63499e7aa3f49e1eaf203b7643c2590eaba654b5",
+            "paper_2509_01190_gb300/csrc/kernels.h": "47cb3d722b2e1c82dff5e4cb066ae28e609907af45c21adc972aa69f769155b7",
         },
     },
 }
