@@ -1106,6 +1106,16 @@ int apply_tail(TileSched& t, int units, const TailPlan& tp) {
   return W > 0 ? units : (parts < units ? parts : units);
 }
 
+// Very deep K and more than two 128-row tiles: whether every 256 x 256 pair tile
+// can be cut into two k-parts that run in one round.  8B down (N 4096, 224
+// k-blocks), 257..512 rows: 47-48 us, against 68 for one wave of whole 128-wide
+// tiles.
+bool pair_parts_fit(int epi, int M, int N, int num_kb, int slots, int cta_slots) {
+  const int tiles = ((M + 255) / 256) * ((N + P_BN - 1) / P_BN);
+  return epi != kEpiSwiGLU && num_kb >= kVeryDeepKb && M > 2 * BM && 2 * slots <= kMaxGemmCtas &&
+         2 * tiles <= slots && 2 * tiles <= cta_slots;
+}
+
 // What the tile plan needs besides the call's shape: how many CTAs (one per
 // SM) and CTA pairs the device runs at once for this epilogue, the split-K
 // workspace, and which tile widths the weight splits and RoPE heads allow.
@@ -1166,7 +1176,9 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
     if (slots > 0 && m_tiles >= 2) {
       const int ptiles = ((m_tiles + 1) / 2) * ((vn + P_BN - 1) / P_BN);
       const double cost = static_cast<double>((ptiles + slots - 1) / slots) * 0.34;
-      if (cost < best - 1e-9) {
+      // (pair tiles that all fit one round in two k-parts: half a wave and the
+      // hand-off, which whole narrow tiles cannot reach)
+      if (cost < best - 1e-9 || pair_parts_fit(epi, in.M, in.N, num_kb, slots, can_split ? cta_slots : 0)) {
         BN = P_BN;
         plan_pairs = true;
         best_tiles = ptiles;
@@ -1289,7 +1301,18 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const TcWeights& W, int epi,
   // most SMs; stream the weights instead
   if (skinny_supported(A, lda, W, epi, p)) return launch_gemm_skinny(A, lda, W, epi, p, s);
   // a few hundred rows: weight band as the 128-row operand, K split over a cluster
-  if (swap_preferred(epi, p.M, p.N, p.K) && swap_supported(A, lda, W, epi, p))
+  // -- except wide weights of very deep K above 320 rows, where the swapped
+  // kernel's row blocks leave one k-block per stage and the pair tiles in two
+  // k-parts take over (8B down: 320 rows 46.1 us swapped and 47.2 in parts, 328
+  // rows 52.6 and 47.1, 512 rows 60.1 and 48.3)
+  const int slots = (pairs_enabled() && bn_ok(P_BN, epi, W, p)) ? pair_slots_for(epi) : 0;
+  // Split-K workspace: slots of BM x 256 fp32 per CTA, four flags each.
+  const bool can_split = p.splitk_ws != nullptr && p.splitk_flags != nullptr;
+  const int cta_slots = can_split ? static_cast<int>(std::min<size_t>(
+                                        p.splitk_ws_elems / (static_cast<size_t>(BM) * 256), kSplitKFlags / 4))
+                                  : 0;
+  const bool parts = p.M > 320 && p.N >= 4096 && pair_parts_fit(epi, p.M, p.N, p.K / BK, slots, cta_slots);
+  if (!parts && swap_preferred(epi, p.M, p.N, p.K) && swap_supported(A, lda, W, epi, p))
     return launch_gemm_swap(A, lda, W, epi, p, s);
   const int vn = epi == kEpiSwiGLU ? 2 * p.N : p.N;
   TilePlanIn in;
@@ -1298,12 +1321,9 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const TcWeights& W, int epi,
   in.N = p.N;
   in.K = p.K;
   in.sms = num_sms();
-  in.slots = (pairs_enabled() && bn_ok(P_BN, epi, W, p)) ? pair_slots_for(epi) : 0;
-  // Split-K workspace: slots of BM x 256 fp32 per CTA, four flags each.
-  in.can_split = p.splitk_ws != nullptr && p.splitk_flags != nullptr;
-  in.cta_slots = in.can_split ? static_cast<int>(std::min<size_t>(p.splitk_ws_elems / (static_cast<size_t>(BM) * 256),
-                                                                   kSplitKFlags / 4))
-                              : 0;
+  in.slots = slots;
+  in.can_split = can_split;
+  in.cta_slots = cta_slots;
   in.bn64 = bn_ok(64, epi, W, p);
   in.bn128 = bn_ok(128, epi, W, p);
   in.bn256 = bn_ok(256, epi, W, p);

@@ -63,6 +63,18 @@ def test_pair_large_1b_shapes(z, name, M, N, K):
     check_linear(out, ref, tol, epi, f"{name} M={M}")
 
 
+# Very deep K in one round of two k-parts per pair tile: the first row count that
+# leaves the swapped kernel (321), three 128-row tiles (the last pair half empty),
+# four, and ragged columns.
+@pytest.mark.parametrize("epi", ["resid", "store"])
+@pytest.mark.parametrize("M,N,K", [(321, 4096, 12288), (384, 4112, 12288), (512, 4096, 14336)])
+def test_pair_two_parts_of_very_deep_k(z, epi, M, N, K):
+    plan, items = z.zsaa_gemm_schedule({"store": 0, "resid": 1}[epi], M, N, K, 64, 152, 76, 256)
+    assert plan[1] == 1 and {it[4] for it in items} == {1, 2}  # pairs; every tile in parts
+    out, ref, tol = linear_case(z, epi, M, N, K, 950 + M)
+    check_linear(out, ref, tol, epi, f"{epi} M={M}")
+
+
 def test_pair_deterministic(z):
     M, N, K = 2048, 2048, 2048
     A = rand_bf16((M, K), 17)
