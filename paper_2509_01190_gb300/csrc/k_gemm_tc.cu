@@ -43,11 +43,11 @@ constexpr int kThreads = 192;
 
 template <int BN>
 struct TcCfg {
-  static constexpr int STAGES = BN >= 256 ? 4 : (BN >= 128 ? 6 : 8);
+  static constexpr int STAGES = BN >= 256 ? 4 : (BN >= 192 ? 5 : (BN >= 128 ? 6 : 8));
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = BN * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int TMEM_COLS = 2 * BN;  // two accumulators
+  static constexpr int TMEM_COLS = BN == 192 ? 512 : 2 * BN;  // two accumulators (a power of two)
   static constexpr size_t SMEM = static_cast<size_t>(STAGES) * STAGE_BYTES + 1024 + 256;
 };
 
@@ -1116,6 +1116,9 @@ bool pair_parts_fit(int epi, int M, int N, int num_kb, int slots, int cta_slots)
          2 * tiles <= slots && 2 * tiles <= cta_slots;
 }
 
+// The one-CTA kernel's time for a k-block of a tile, every SM streaming, in us.
+double step_us(int BN) { return BN == 256 ? 0.36 : (BN == 192 ? 0.30 : 0.27); }
+
 // What the tile plan needs besides the call's shape: how many CTAs (one per
 // SM) and CTA pairs the device runs at once for this epilogue, the split-K
 // workspace, and which tile widths the weight splits and RoPE heads allow.
@@ -1126,7 +1129,9 @@ struct TilePlanIn {
   bool can_split;  // a split-K workspace and flags were given
   int cta_slots;   // its partial slots (BM x 256 fp32, four flags each)
   bool bn64, bn128, bn256;
-  bool width_ok(int BN) const { return BN == 64 ? bn64 : (BN == 128 ? bn128 : (BN == 256 && bn256)); }
+  bool width_ok(int BN) const {
+    return BN == 64 ? bn64 : (BN == 128 ? bn128 : (BN == 192 ? epi == kEpiSwiGLU : BN == 256 && bn256));
+  }
 };
 
 // The plan: the one-CTA kernel's tile width, grid and work split, and, when
@@ -1152,7 +1157,7 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
   if (num_kb >= kDeepKb) {
     // Deep K (>= 64 k-blocks: every 8B projection, the 1B down projection):
     // the plan with the least waves x cost of one k-block step
-    // -- one-CTA tiles 128 or 256 wide, or 256 x 256 tiles on CTA pairs (only
+    // -- one-CTA tiles 128, 192 or 256 wide, or 256 x 256 tiles on CTA pairs (only
     // with two or more 128-row tiles: a lone one would leave half of each pair
     // tile empty); then its ragged last wave possibly cut into aligned k-parts
     // (tail_plan).  The step costs are GB300 graph-timed averages over the 1B
@@ -1161,12 +1166,17 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
     // Narrow tiles win only while they still fit one wave (8B QKV at 316
     // rows: 25.2 us against 30.1 on pairs); pairs win while they add no wave
     // (8B O at 744 rows: 27.7 us against 33.0 on the swapped kernel).
+    // SwiGLU of up to 384 rows (one to three row tiles, where the weight stream
+    // and the last wave decide) also has 192-wide tiles, 0.30 us: 8B gate/up is
+    // 150 of them per row tile, a wave of the 152 SMs each.  Against 256-wide
+    // tiles and pairs: 17..128 rows 46 -> 43 us, 129..256 rows 56 -> 51.5,
+    // 257..384 rows 71 -> 68.5.  (More row tiles: pairs re-read less from L2.)
     double best = 1e30;
     int best_tiles = 0;
-    for (int cand : {128, 256}) {
-      if (!in.width_ok(cand)) continue;
+    for (int cand : {128, 192, 256}) {
+      if (!in.width_ok(cand) || (cand == 192 && (m_tiles > 3 || num_kb >= kVeryDeepKb))) continue;
       const int tiles = m_tiles * ((vn + cand - 1) / cand);
-      const double cost = static_cast<double>((tiles + sms - 1) / sms) * (cand == 256 ? 0.36 : 0.27);
+      const double cost = static_cast<double>((tiles + sms - 1) / sms) * step_us(cand);
       if (cost < best - 1e-9) {
         best = cost;
         BN = cand;
@@ -1187,7 +1197,7 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
     if (BN != 0 && num_kb >= kVeryDeepKb) {
       plan_tp = plan_pairs ? tail_plan(best_tiles, slots, num_kb, 0.34, can_split && 2 * slots <= kMaxGemmCtas,
                                        cta_slots / 2)
-                           : tail_plan(best_tiles, sms, num_kb, BN == 256 ? 0.36 : 0.27,
+                           : tail_plan(best_tiles, sms, num_kb, step_us(BN),
                                        can_split && sms <= kMaxGemmCtas, cta_slots);
     }
   }
@@ -1358,6 +1368,7 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const TcWeights& W, int epi,
   if (pairs > 0) return dispatch_pair(epi, maps, n1, n2, p, ps, pairs, s);
   switch (BN) {
     case 256: return dispatch_epi<256>(epi, maps, n1, n2, p, ts, grid, s);
+    case 192: return run_tc<192, kEpiSwiGLU>(maps, n1, n2, p, ts, grid, s);
     case 128: return dispatch_epi<128>(epi, maps, n1, n2, p, ts, grid, s);
     default: return dispatch_epi<64>(epi, maps, n1, n2, p, ts, grid, s);
   }

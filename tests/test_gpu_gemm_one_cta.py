@@ -45,6 +45,17 @@ def test_one_cta_tiled_paths(zlib):
     assert r.stdout.count("ok ") == len(CASES), r.stdout
 
 
+# 192-wide SwiGLU tiles (deep K, up to three row tiles, one wave of them per row
+# tile): one, two and three row tiles, and a last column tile of 64 or 16 gate rows.
+@pytest.mark.parametrize("M,N,K", [(33, 9760, 4096), (129, 9808, 4096), (300, 14336, 4096)])
+def test_192_wide_swiglu_tiles(zlib, M, N, K):
+    need_gpu()
+    plan, _ = zlib.zsaa_gemm_schedule(2, M, N, K, 64, 152, 76, 256)
+    assert plan[0] == 192 and plan[1] == 0
+    out, ref, tol = linear_case(zlib, "swiglu", M, N, K, 1450 + M)
+    check_linear(out, ref, tol, "swiglu", f"M={M} N={N}")
+
+
 if __name__ == "__main__":
     sys.path.insert(0, ROOT)
     _run_cases()
