@@ -11,8 +11,8 @@
 // column mass: C[b,g,j] = sum over heads h of group g, queries i >= j, of
 //   P[i,j], recomputed from q, k and lse2 (no N x N matrix is stored).
 //
-// bf16 path (the masked mode's attention, and calls without a status word; the
-// others run on tcgen05): FlashAttention-style tiles on mma.sync m16n8k16 (64 queries x 64
+// bf16 path (short sequences, the masked mode, and calls without a status word;
+// the others run on tcgen05): FlashAttention-style tiles on mma.sync m16n8k16 (64 queries x 64
 // keys per step, 4 warps x 16 rows), online softmax in fp32; the probabilities
 // enter P V as a hi/lo pair of bf16 matrices.  The column-mass
 // pass sweeps key blocks outer / query blocks inner so each CTA owns its
@@ -50,13 +50,14 @@ __device__ __forceinline__ void load_tile64(uint32_t sbase, const bf16* g, size_
 
 template <int HD>
 __global__ void __launch_bounds__(128)
-    attn_fwd_bf16_kernel(const bf16* __restrict__ qkv, int N, int Hq, int Hkv,
+    attn_fwd_bf16_kernel(const bf16* __restrict__ qkv, int Ns, int Hq, int Hkv,
                          bf16* __restrict__ out, float* __restrict__ lse2, float scale_log2,
-                         int causal, const uint8_t* __restrict__ key_alive) {
+                         int causal, const uint8_t* __restrict__ key_alive, const int* __restrict__ cu) {
   pdl_trigger();
   pdl_wait();
   qkv = after_wait(qkv);
   key_alive = after_wait(key_alive);
+  cu = after_wait(cu);
   constexpr int ROWB = HD * 2;
   constexpr int TILE = 64 * ROWB;
   extern __shared__ __align__(128) uint8_t sm[];
@@ -64,9 +65,13 @@ __global__ void __launch_bounds__(128)
   const uint32_t sK0 = sQ + TILE, sV0 = sQ + 3 * TILE;  // K: 2 buffers, V: 2 buffers
 
   const int qb = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const size_t row0 = static_cast<size_t>(b) * N;
+  // fixed length: N = Ns rows per sequence; packed variable length: this
+  // sequence's rows [cu[b], cu[b+1]) (Ns = the longest: grid and lse stride)
+  const size_t row0 = cu ? static_cast<size_t>(cu[b]) : static_cast<size_t>(b) * Ns;
+  const int N = cu ? cu[b + 1] - cu[b] : Ns;
+  if (qb * 64 >= N) return;
   // masked mode (Appendix B): keys whose flag is 0 are hidden from every query
-  const uint8_t* ka = key_alive ? key_alive + static_cast<size_t>(b) * N : nullptr;
+  const uint8_t* ka = key_alive ? key_alive + static_cast<size_t>(b) * Ns : nullptr;
   const int g = h / (Hq / Hkv);
   const size_t ld = static_cast<size_t>(Hq + 2 * Hkv) * HD;
   const bf16* base = qkv + row0 * ld;
@@ -207,7 +212,7 @@ __global__ void __launch_bounds__(128)
     for (int nt = 0; nt < HD / 8; ++nt)
       *reinterpret_cast<uint32_t*>(orow + nt * 8 + 2 * tig) =
           pack_bf16x2(o[nt][0] * inv_lo, o[nt][1] * inv_lo);
-    if (tig == 0) lse2[(static_cast<size_t>(b) * Hq + h) * N + i_lo] = m_lo + log2f(l_lo);
+    if (tig == 0) lse2[(static_cast<size_t>(b) * Hq + h) * Ns + i_lo] = m_lo + log2f(l_lo);
   }
   if (i_hi < N) {
     bf16* orow = out + (row0 + i_hi) * ldo + h * HD;
@@ -215,7 +220,7 @@ __global__ void __launch_bounds__(128)
     for (int nt = 0; nt < HD / 8; ++nt)
       *reinterpret_cast<uint32_t*>(orow + nt * 8 + 2 * tig) =
           pack_bf16x2(o[nt][2] * inv_hi, o[nt][3] * inv_hi);
-    if (tig == 0) lse2[(static_cast<size_t>(b) * Hq + h) * N + i_hi] = m_hi + log2f(l_hi);
+    if (tig == 0) lse2[(static_cast<size_t>(b) * Hq + h) * Ns + i_hi] = m_hi + log2f(l_hi);
   }
 }
 
@@ -479,9 +484,23 @@ __global__ void colmass_f32_kernel(const float* __restrict__ qkv, const float* _
 
 }  // namespace
 
+// Short sequences: a CTA of the mma.sync kernel holds 64 queries and 64 keys and
+// ends after one step, where the tcgen05 kernel's items are 128 wide and run a
+// chain of MMAs, softmax and epilogue each.  Measured (tcgen05 / mma.sync, us):
+// 32 heads of 64 over 8, N = 48: 1 sequence 5.3 / 3.2, 19: 9.7 / 7.7, 64: 27.7 /
+// 19.1; N = 64 and 64 sequences 28.7 / 19.9; N = 80 (two steps a row) 30.1 / 49.3.
+// Heads of 128: N = 64, 8 sequences of 32 heads 7.4 / 6.2, 19: 11.5 / 11.5, 64:
+// 33.1 / 37.9, so up to 512 heads in all.  With lengths that differ the mean
+// decides, up to twice that length (19 of 12..71: 18.2 / 12.5 with events).
+// (its grid holds 65535 sequences, its copies need aligned rows)
+bool attention_short(const void* qkv, int hd, int B, int N, long long rows, int Hq) {
+  return N <= 128 && rows <= 64LL * B && (hd == 64 || static_cast<long long>(B) * Hq <= 512) && B <= 65535 &&
+         (reinterpret_cast<uintptr_t>(qkv) & 15) == 0;
+}
+
 cudaError_t launch_attention(int dtype, const void* qkv, int B, int N, int Hq, int Hkv, int hd,
-                             void* out, float* lse, int causal, cudaStream_t s, const uint8_t* key_alive) {
-  if (key_alive != nullptr && dtype != ZSAA_BF16) return cudaErrorInvalidValue;
+                             void* out, float* lse, int causal, cudaStream_t s, const uint8_t* key_alive, const int* cu) {
+  if ((key_alive != nullptr || cu != nullptr) && dtype != ZSAA_BF16) return cudaErrorInvalidValue;
   const float scale_log2 = kLog2e / sqrtf(static_cast<float>(hd));
   if (dtype == ZSAA_F32 && attention_f32_tiled(qkv, hd))
     return launch_attention_f32_tiled(static_cast<const float*>(qkv), B, N, Hq, Hkv, hd, static_cast<float*>(out),
@@ -499,14 +518,14 @@ cudaError_t launch_attention(int dtype, const void* qkv, int B, int N, int Hq, i
     const cudaError_t e = set_smem_limit_once(once, attn_fwd_bf16_kernel<64>, smem);
     if (e != cudaSuccess) return e;
     ZSAA_LAUNCH(attn_fwd_bf16_kernel<64>, dim3(grid), dim3(128), smem, s, static_cast<const bf16*>(qkv), N, Hq, Hkv,
-                                                      static_cast<bf16*>(out), lse, scale_log2, causal, key_alive);
+                                                      static_cast<bf16*>(out), lse, scale_log2, causal, key_alive, cu);
   } else if (hd == 128) {
     const int smem = 5 * 64 * 256;
     static OncePerDevice once;
     const cudaError_t e = set_smem_limit_once(once, attn_fwd_bf16_kernel<128>, smem);
     if (e != cudaSuccess) return e;
     ZSAA_LAUNCH(attn_fwd_bf16_kernel<128>, dim3(grid), dim3(128), smem, s, static_cast<const bf16*>(qkv), N, Hq, Hkv,
-                                                       static_cast<bf16*>(out), lse, scale_log2, causal, key_alive);
+                                                       static_cast<bf16*>(out), lse, scale_log2, causal, key_alive, cu);
   } else {
     return cudaErrorInvalidValue;
   }

@@ -168,11 +168,14 @@ cudaError_t launch_gemm_f32(const float* A, int lda, const TcWeights& W, int epi
 bool attention_pp_supported(int dtype, int hd, int Hq, int Hkv, const uint8_t* key_alive, int* status);
 cudaError_t launch_attention_pp(const void* qkv, int B, int N, int Hq, int Hkv, int hd, void* out, float* lse,
                                 int causal, int* status, cudaStream_t s, const int* cu = nullptr, int rows = 0);
+// Whether sequences of N rows at most, `rows` in all, are short enough that the
+// mma.sync kernel below is the faster one.
+bool attention_short(const void* qkv, int hd, int B, int N, long long rows, int Hq);
 // causal = 0: bidirectional (Eq. 1 with M = 0); the column-mass kernels below
-// take the same flag.
+// take the same flag.  cu as above (bf16).
 cudaError_t launch_attention(int dtype, const void* qkv, int B, int N, int Hq, int Hkv, int hd,
                              void* out, float* lse, int causal, cudaStream_t s,
-                             const uint8_t* key_alive = nullptr);
+                             const uint8_t* key_alive = nullptr, const int* cu = nullptr);
 // key_alive (bf16, fixed length): [B, N] flags of the masked mode; keys with 0
 // are hidden from every query.
 // fp32 tiled kernels (k_attn_f32.cu): heads of 32, 64 or 128 dims, 16-byte

@@ -627,7 +627,7 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
     {
       const double pairs = static_cast<double>(B) * Hq * n_pairs(N);
       TRACE("attention", 4.0 * pairs * hd, Md * (m->ld_qkv + m->dq) * es + static_cast<double>(B) * Hq * N * 4.0);
-      if (attention_pp_supported(dt, hd, Hq, Hkv, nullptr, m->status)) {
+      if (attention_pp_supported(dt, hd, Hq, Hkv, nullptr, m->status) && !attention_short(m->qkv, hd, B, N, M, Hq)) {
         ZCK(launch_attention_pp(m->qkv, B, N, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s));
       } else {
         ZCK(launch_attention(dt, m->qkv, B, N, Hq, Hkv, hd, m->attn, m->lse, causal, s));
@@ -914,7 +914,8 @@ zsaa_status run_forward_masked(zsaa_model* m, const int32_t* tok, int B, int L, 
     }
     {
       TRACE("attention", 4.0 * pairs * hd, Md * (m->ld_qkv + m->dq) * es + static_cast<double>(B) * Hq * L * 4.0);
-      if (reactivate && attention_pp_supported(dt, hd, Hq, Hkv, nullptr, m->status)) {  // nothing is hidden
+      if (reactivate && attention_pp_supported(dt, hd, Hq, Hkv, nullptr, m->status) &&
+          !attention_short(m->qkv, hd, B, L, static_cast<long long>(B) * L, Hq)) {  // nothing is hidden
         ZCK(launch_attention_pp(m->qkv, B, L, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s));
       } else {
         ZCK(launch_attention(dt, m->qkv, B, L, Hq, Hkv, hd, m->attn, m->lse, causal, s,
@@ -1152,7 +1153,10 @@ zsaa_status run_forward_varlen(zsaa_model* m, const int32_t* tok, const int32_t*
         pairs += causal ? nb * (nb + 1) / 2.0 : nb * nb;
       }
       TRACE("attention", 4.0 * pairs * Hq * hd, Md * (m->ld_qkv + m->dq) * es + static_cast<double>(B) * Hq * Nm * 4.0);
-      ZCK(launch_attention_pp(m->qkv, B, Nm, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s, cu_dev(li), M));
+      if (attention_short(m->qkv, hd, B, Nm, M, Hq))
+        ZCK(launch_attention(dt, m->qkv, B, Nm, Hq, Hkv, hd, m->attn, m->lse, causal, s, nullptr, cu_dev(li)));
+      else
+        ZCK(launch_attention_pp(m->qkv, B, Nm, Hq, Hkv, hd, m->attn, m->lse, causal, m->status, s, cu_dev(li), M));
     }
     // O-projection beside the column mass and selection (see run_forward)
     const bool fork = !m->tracing && prunes(c, l) && rows[l] < M && Nm <= kSelectPartsMaxN;
@@ -1898,7 +1902,8 @@ zsaa_status zsaa_op_attention_ex(const void* qkv, int B, int N, int Hq, int Hkv,
   if (dtype == ZSAA_F32 && (hd < 1 || hd > 128)) return fail(ZSAA_ERR_UNSUPPORTED, "f32 attention needs hd <= 128");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int* status = shared_status();
-  if (attention_pp_supported(dtype, hd, Hq, Hkv, nullptr, status)) {
+  if (attention_pp_supported(dtype, hd, Hq, Hkv, nullptr, status) &&
+      !attention_short(qkv, hd, B, N, static_cast<long long>(B) * N, Hq)) {
     ZCK(launch_attention_pp(qkv, B, N, Hq, Hkv, hd, out, lse, causal ? 1 : 0, status, s));
     return ZSAA_OK;
   }

@@ -9,7 +9,9 @@ import torch
 from oracle import zsaa_oracle as O
 from paper_2509_01190_gb300 import inputs as I
 from tests.helpers import bf16_ulp_close, need_gpu
+from tests.test_gpu_forward import SMALL_BF16, SMALL_BF16_128
 from tests.test_gpu_ops import _np, _oracle_attention, _qkv
+from tests.test_gpu_varlen import check_varlen, run_varlen_case
 
 pytestmark = pytest.mark.gpu
 
@@ -47,6 +49,24 @@ def test_attention_tiles(z, B, N, Hq, Hkv, hd, causal):
     assert np.all(bf16_ulp_close(got, ref_b, 1, 1e-5 * np.abs(ref_o).max(axis=-1, keepdims=True)))
     assert np.mean(got == ref_b) > 0.95
     np.testing.assert_allclose(_np(lse), ref_lse, rtol=1e-5, atol=1e-4)
+
+
+# Both sides of the lines between this kernel and the mma.sync one of short
+# sequences: 64 rows, and for heads of 128 dims 512 heads in all.
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("B,N,Hq,Hkv,hd", [(3, 63, 4, 2, 64), (3, 64, 4, 2, 64), (3, 65, 4, 2, 64), (64, 48, 32, 8, 64),
+                                           (16, 64, 32, 8, 128), (17, 64, 32, 8, 128), (128, 5, 4, 4, 128),
+                                           (129, 5, 4, 4, 128)])
+def test_attention_of_short_sequences(z, B, N, Hq, Hkv, hd, causal):
+    test_attention_tiles(z, B, N, Hq, Hkv, hd, causal)
+
+
+# Packed lengths of at most 64 rows on average and up to 128 run on the mma.sync
+# kernel, longer ones (mean 65, or one of 129) on this.
+@pytest.mark.parametrize("lengths", [[128, 1, 60, 30, 64], [64, 64, 64], [64, 64, 67], [129, 1, 20, 30]])
+def test_packed_short_sequences(z, lengths):
+    for shape in (SMALL_BF16, SMALL_BF16_128):
+        check_varlen(run_varlen_case(z, shape, lengths, 1.5), shape)
 
 
 # An output that allows 16-byte but not 32-byte stores gives the same values.
