@@ -861,6 +861,7 @@ cudaError_t launch_rows_norm(int dtype, const void* src, const int32_t* tok, int
                              int d, const void* w, float eps, void* h_out, void* x_out,
                              int32_t* pos_out, int* status, cudaStream_t s, const int* cu_src,
                              const int* cu_dst, int nseq) {
+  if (!rows_norm_supported(dtype, d)) return cudaErrorInvalidValue;  // the largest Q would leave columns out
   return norm_dispatch(dtype, d, [&](auto t, int vec, auto q) -> cudaError_t {
     using T = decltype(t);
     constexpr int Q = decltype(q)::value;

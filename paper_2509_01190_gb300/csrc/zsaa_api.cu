@@ -1464,10 +1464,17 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
     p.norm_eps = c.rms_eps;
   };
 #define TRACE(name, fl, by) TraceScope trace_scope_(m, name, fl, by, s)
-  {
+  if (rows_norm_supported(c.dtype, d)) {
     TRACE("embed_norm", 0.0, Bd * (3.0 * d * es + 8.0));
     ZCK(launch_rows_norm(c.dtype, m->embed, tok, c.vocab, 1, nullptr, 0, 0, nullptr, B, d,
                          LW(m, 0, kAttnNorm), c.rms_eps, h, m->x, m->pos[0], m->status, s));
+  } else {  // wider rows than a warp's registers hold
+    {
+      TRACE("embed", 0.0, Bd * (2.0 * d * es + 8.0));
+      ZCK(launch_embed(c.dtype, m->embed, tok, B, 1, c.vocab, d, h, m->pos[0], m->status, s));
+    }
+    TRACE("rmsnorm", 0.0, 2.0 * Bd * d * es);
+    ZCK(launch_rmsnorm(c.dtype, h, LW(m, 0, kAttnNorm), B, d, c.rms_eps, m->x, s));
   }
   for (int li = 0; li < c.n_layers; ++li) {
     const bool in_norm = fuse && li > 0;  // layer 0's rows come normed from the embedding

@@ -30,3 +30,20 @@ def test_decode_rows(z, shape, B, L, T, accel):
     for t in range(T):
         mx, mean = logits_report(r["step_logits"][:, t], r["ores"]["logits"][:, t])
         assert mx <= BF16_MAX_ABS and mean <= BF16_MEAN_ABS, (t, mx, mean)
+
+
+# Residual rows of more than 512 16-byte vectors (d 4096): the step embeds and norms
+# them in kernels of their own, in front of the folded projections (up to 16
+# sequences, d 8192) and of the plain ones.  A logit is a sum of d products of a
+# unit-RMS row and weights of std 0.02, so its error grows with its own size: the
+# bound is the one of chained forwards, 2^-7 of the logits' std per layer (mean) and
+# eight times that (max).
+@pytest.mark.parametrize("d,B", [(4160, 2), (5120, 16), (5120, 17), (8192, 3), (8256, 2)])
+def test_decode_of_wide_rows(z, d, B):
+    shape = I.ModelShape("wide-bf16", 2, d, 4, 2, 64, 256, 1008)
+    r = run_generate(z, shape, B, 20, 3, 1.5)
+    for got, ref in [(r["prefill_logits"], r["ores"]["prefill"]["logits"][:, -1])] + [
+            (r["step_logits"][:, t], r["ores"]["logits"][:, t]) for t in range(3)]:
+        mx, mean = logits_report(got, ref)
+        floor = 2.0 ** -7 * shape.n_layers ** 0.5 * ref.std()
+        assert mean <= floor and mx <= 8 * floor, (mx, mean, floor)
