@@ -93,7 +93,10 @@ typedef struct {
  *   attn_norm [d], wq [Hq*hd, d], wk [Hkv*hd, d], wv [Hkv*hd, d],
  *   wo [d, Hq*hd], mlp_norm [d], wg [F, d], wu [F, d], wd [d, F].
  * embed is [vocab, d]; final_norm [d]; head is [vocab, d] (may equal embed)
- * or [n_classes, d].  The pointer array itself is copied at create time. */
+ * or [n_classes, d].  The pointer array itself is copied at create time.
+ * Layer weights start on 16-byte boundaries (checked at create time), as does
+ * embed for every call that reads token ids (checked there) and a bf16 LM head;
+ * final_norm, a float32 head and a classifier's may start at any element. */
 typedef struct {
   const void* embed;
   const void* const* layers;

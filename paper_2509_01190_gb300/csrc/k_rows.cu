@@ -760,14 +760,16 @@ cudaError_t launch_embed(int dtype, const void* E, const int32_t* tok, int rows,
   return cudaGetLastError();
 }
 
-bool rows_norm_supported(int dtype, int d) {
+bool rows_norm_supported(int dtype, int d, const void* w) {
   const int bytes = d * (dtype == ZSAA_BF16 ? 2 : 4);
-  return bytes % 16 == 0 && bytes / 16 <= 32 * kMaxVecPerLane;
+  return bytes % 16 == 0 && bytes / 16 <= 32 * kMaxVecPerLane && (reinterpret_cast<uintptr_t>(w) & 15) == 0;
 }
 
 cudaError_t launch_rmsnorm(int dtype, const void* h, const void* w, int rows, int d, float eps,
                            void* x, cudaStream_t s) {
-  if (rows_norm_supported(dtype, d)) {
+  // (the rows are the library's own buffers; the weights, of the final norm, may be
+  // any view of the caller's: element by element where they allow no 16-byte reads)
+  if (rows_norm_supported(dtype, d, w)) {
     return norm_dispatch(dtype, d, [&](auto t, int vec, auto q) -> cudaError_t {
       using T = decltype(t);
       constexpr int Q = decltype(q)::value;
@@ -776,7 +778,7 @@ cudaError_t launch_rmsnorm(int dtype, const void* h, const void* w, int rows, in
                   vec, eps, static_cast<uint4*>(x));
       return cudaGetLastError();
     });
-  } else if (dtype == ZSAA_BF16 && d % 8 == 0) {
+  } else if (dtype == ZSAA_BF16 && d % 8 == 0 && (reinterpret_cast<uintptr_t>(w) & 15) == 0) {
     ZSAA_LAUNCH(rmsnorm_bf16_vec_kernel, dim3(row_blocks(rows)), dim3(32 * kWarpsPerBlock), 0, s, 
         static_cast<const uint4*>(h), static_cast<const uint4*>(w), rows, d / 8, eps,
         static_cast<uint4*>(x));
@@ -861,7 +863,8 @@ cudaError_t launch_rows_norm(int dtype, const void* src, const int32_t* tok, int
                              int d, const void* w, float eps, void* h_out, void* x_out,
                              int32_t* pos_out, int* status, cudaStream_t s, const int* cu_src,
                              const int* cu_dst, int nseq) {
-  if (!rows_norm_supported(dtype, d)) return cudaErrorInvalidValue;  // the largest Q would leave columns out
+  // (the largest Q would leave columns of a wider row out)
+  if (!rows_norm_supported(dtype, d, w)) return cudaErrorInvalidValue;
   return norm_dispatch(dtype, d, [&](auto t, int vec, auto q) -> cudaError_t {
     using T = decltype(t);
     constexpr int Q = decltype(q)::value;

@@ -34,9 +34,10 @@ cudaError_t launch_select_parts(const float* parts, int n_qc, int B, int G, int 
 // Embedding when idx == nullptr (rows = B*L, source row tok[r] of E);
 // otherwise compaction (rows = B*k, source row b*N + idx[r] of h).
 // Rows of whole 16-byte vectors, at most 512 of them (bf16: d % 8 == 0 and
-// d <= kRowsNormMaxD; float: d % 4 == 0 and half of that); others are refused.
+// d <= kRowsNormMaxD; float: d % 4 == 0 and half of that), norm weights w on a
+// 16-byte boundary; others are refused.
 constexpr int kRowsNormMaxD = 8 * 32 * 16;
-bool rows_norm_supported(int dtype, int d);
+bool rows_norm_supported(int dtype, int d, const void* w = nullptr);
 // Variable length: cu_dst (offsets of the written rows; nseq sequences) gives
 // the sequence of a row and, for the embedding, pos = r - cu_dst[b]; cu_src
 // (offsets of the source rows) places compaction index j at row cu_src[b] + j.

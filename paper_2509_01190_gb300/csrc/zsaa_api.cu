@@ -47,6 +47,8 @@ zsaa_status fail(zsaa_status st, const char* fmt, ...) {
                   __FILE__, __LINE__);                                                   \
   } while (0)
 
+bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
 // ---------------------------------------------------------------- planner
 
 bool prunes(const zsaa_config& c, int layer) { return (c.prune_mask >> (layer - 1)) & 1ull; }
@@ -510,6 +512,7 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
   const bool from_hidden = opts && opts->hidden_in;
   if ((!from_hidden && tok == nullptr) || logits == nullptr)
     return fail(ZSAA_ERR_INVALID_ARG, "null token or logits pointer");
+  if (!from_hidden && !aligned16(m->embed)) return fail(ZSAA_ERR_INVALID_ARG, "embed not 16-byte aligned");
   if (B < 1 || B > m->max_B || L < 1 || L > m->max_L)
     return fail(ZSAA_ERR_INVALID_ARG, "B=%d L=%d outside [1,%d] x [1,%d]", B, L, m->max_B, m->max_L);
   const int first = from_hidden ? opts->first_layer : 1;
@@ -769,7 +772,7 @@ zsaa_status run_forward(zsaa_model* m, const int32_t* tok, int B, int L, double 
   if (opts && opts->hidden_out)
     ZCK(cudaMemcpyAsync(opts->hidden_out, m->h[cur], M * d * m->esz, cudaMemcpyDeviceToDevice, s));
   if (kc != nullptr) {  // next-token logits: final norm and LM head of the last kept row
-    if (fuse_norm) {
+    if (rows_norm_supported(dt, d, m->final_norm)) {
       TRACE("gather_norm", 0.0, static_cast<double>(B) * (3.0 * d * es + 12.0));
       ZCK(launch_rows_norm(dt, m->h[cur], nullptr, 0, 0, kc->last_idx, N, 1, m->pos[cur], B, d,
                            m->final_norm, c.rms_eps, m->h[cur ^ 1], m->x, m->pos[cur ^ 1],
@@ -859,6 +862,7 @@ zsaa_status run_forward_masked(zsaa_model* m, const int32_t* tok, int B, int L, 
   if (c.dtype != ZSAA_BF16 || d % 8 != 0 || d > kRowsNormMaxD)
     return fail(ZSAA_ERR_UNSUPPORTED, "the masked mode needs a bf16 model with d_model <= %d", kRowsNormMaxD);
   if (tok == nullptr || logits == nullptr) return fail(ZSAA_ERR_INVALID_ARG, "null token or logits pointer");
+  if (!aligned16(m->embed)) return fail(ZSAA_ERR_INVALID_ARG, "embed not 16-byte aligned");
   if (B < 1 || B > m->max_B || L < 1 || L > m->max_L)
     return fail(ZSAA_ERR_INVALID_ARG, "B=%d L=%d outside [1,%d] x [1,%d]", B, L, m->max_B, m->max_L);
   if (L > kSelectPartsMaxN) return fail(ZSAA_ERR_UNSUPPORTED, "the masked mode needs L <= %d", kSelectPartsMaxN);
@@ -1019,15 +1023,22 @@ zsaa_status run_forward_masked(zsaa_model* m, const int32_t* tok, int B, int L, 
   const int nf = sched[n];
   void* hf = h;
   const int32_t* posf = m->pos[0];
+  const bool fuse_final = rows_norm_supported(dt, d, m->final_norm);
   if (kept != nullptr) {
-    TRACE("gather_norm", 0.0, static_cast<double>(B) * nf * (3.0 * d * es + 12.0));
-    ZCK(launch_rows_norm(dt, h, nullptr, 0, 0, kept, L, nf, m->pos[0], B * nf, d, m->final_norm,
-                         c.rms_eps, m->h[1], m->x, m->pos[1], m->status, s));
+    if (fuse_final) {
+      TRACE("gather_norm", 0.0, static_cast<double>(B) * nf * (3.0 * d * es + 12.0));
+      ZCK(launch_rows_norm(dt, h, nullptr, 0, 0, kept, L, nf, m->pos[0], B * nf, d, m->final_norm,
+                           c.rms_eps, m->h[1], m->x, m->pos[1], m->status, s));
+    } else {
+      TRACE("gather", 0.0, static_cast<double>(B) * nf * (2.0 * d * es + 12.0));
+      ZCK(launch_gather(h, B, L, nf, static_cast<int>(d * m->esz), kept, m->h[1], m->pos[0], m->pos[1], m->status, s));
+    }
     hf = m->h[1];
     posf = m->pos[1];
-  } else if (c.n_classes == 0) {
+  }
+  if (c.n_classes == 0 && (kept == nullptr || !fuse_final)) {
     TRACE("rmsnorm", 0.0, 2.0 * static_cast<double>(B) * nf * d * es);
-    ZCK(launch_rmsnorm(dt, h, m->final_norm, B * nf, d, c.rms_eps, m->x, s));
+    ZCK(launch_rmsnorm(dt, hf, m->final_norm, B * nf, d, c.rms_eps, m->x, s));
   }
   if (c.n_classes > 0) {
     TRACE("cls_head", 2.0 * B * d * c.n_classes, (static_cast<double>(B) * d + static_cast<double>(c.n_classes) * d) * es);
@@ -1065,6 +1076,7 @@ zsaa_status run_forward_varlen(zsaa_model* m, const int32_t* tok, const int32_t*
     return fail(ZSAA_ERR_UNSUPPORTED, "variable-length batches need a bf16 model with d_model <= %d", kRowsNormMaxD);
   if (tok == nullptr || logits == nullptr || lengths == nullptr)
     return fail(ZSAA_ERR_INVALID_ARG, "null token, lengths or logits pointer");
+  if (!aligned16(m->embed)) return fail(ZSAA_ERR_INVALID_ARG, "embed not 16-byte aligned");
   if (B < 1 || B > m->max_B) return fail(ZSAA_ERR_INVALID_ARG, "B=%d outside [1,%d]", B, m->max_B);
   if (opts && (opts->hidden_out || opts->n_layers_run || opts->hidden_in || opts->pos_in ||
                opts->first_layer || opts->plan_L))
@@ -1456,7 +1468,7 @@ zsaa_status run_decode(zsaa_model* m, zsaa_cache* kc, const int32_t* tok, float*
   // leave the rows' sums of squares and the next projection norms the rows
   // itself, so only the embedding's norm is a kernel of its own; the head's
   // kernel steps the position.
-  const bool fuse = skinny_norm_supported(B, d) && reinterpret_cast<uintptr_t>(m->head) % 16 == 0;
+  const bool fuse = skinny_norm_supported(B, d) && aligned16(m->head) && aligned16(m->final_norm);
   float* ss[2] = {kc->norm_ss, kc->norm_ss + d};  // after the attention branch, after the MLP branch
   auto normed = [&](GemmParams& p, const void* w, const float* sums) {
     p.norm_w = w;
@@ -1658,7 +1670,7 @@ zsaa_status zsaa_model_create(const zsaa_config* cfg, const zsaa_weights* w, int
   for (int i = 0; i < cfg->n_layers * 9; ++i) {
     const void* p = w->layers[i];
     if (p == nullptr) return fail(ZSAA_ERR_INVALID_ARG, "null layer weight %d", i);
-    if (reinterpret_cast<uintptr_t>(p) % 16) return fail(ZSAA_ERR_INVALID_ARG, "layer weight %d not 16-byte aligned", i);
+    if (!aligned16(p)) return fail(ZSAA_ERR_INVALID_ARG, "layer weight %d not 16-byte aligned", i);
   }
   const long long rows = static_cast<long long>(max_B) * max_L;
   if (rows > (1LL << 30)) return fail(ZSAA_ERR_INVALID_ARG, "max_B*max_L too large");
