@@ -96,7 +96,10 @@ typedef struct {
  * or [n_classes, d].  The pointer array itself is copied at create time.
  * Layer weights start on 16-byte boundaries (checked at create time), as does
  * embed for every call that reads token ids (checked there) and a bf16 LM head;
- * final_norm, a float32 head and a classifier's may start at any element. */
+ * final_norm, a float32 head and a classifier's may start at any element.
+ * Weights may be changed between calls: a forward or decode step reads them
+ * after everything enqueued before it on its stream, other calls of this
+ * library included, has ended. */
 typedef struct {
   const void* embed;
   const void* const* layers;
@@ -362,9 +365,10 @@ zsaa_status zsaa_score_select_noalloc(const void* hidden, int B, int L, int d, i
  * split-K partials also added in a fixed order), ZSAA_F32 the fp32 CUDA-core
  * GEMM.  ZSAA_GEMM_PAIRS=0 in the environment (read once per process) keeps
  * the tiled GEMM on one CTA, a diagnostic switch with the same results up to
- * summation order.  The bf16 kernels start reading W before the
- * previous library kernel on the stream has finished: W and W2 must not be
- * written by that kernel.  epilogue:
+ * summation order.  The bf16 kernels start reading W while earlier
+ * library kernels on the stream may still run: W and W2 must not be written by
+ * a zsaa_op_* call since the last copy or kernel of the caller's on the stream
+ * or synchronisation.  epilogue:
  *   0 store (out has dtype; bf16 rounds once),
  *   1 residual: out = resid + acc (resid may alias out),
  *   2 SwiGLU: out[M,N] = silu(A W^T) * (A W2^T), W and W2 both [N,K],

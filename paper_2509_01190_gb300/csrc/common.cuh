@@ -56,7 +56,7 @@ enum : int { kStatusTimeout = 1, kStatusBadIndex = 2 };
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
 
 // Programmatic dependent launch: every kernel of the library is launched with
-// launch_pdl, lets the next kernel in the stream start its prologue at once
+// launch_kernel, lets the next kernel in the stream start its prologue at once
 // (pdl_trigger), and waits for the previous kernel's results (pdl_wait)
 // before touching global data another kernel writes or reads.  Without the
 // launch attribute both are no-ops.
@@ -77,9 +77,13 @@ __device__ __forceinline__ T* after_wait(T* p) {
   return p;
 }
 
+// early = false: the kernel starts only when everything before it on the stream
+// has ended.  The first kernel of a forward or decode step is launched so, because
+// the kernels after it read weights before their own wait: weights that an earlier
+// call of the library on the stream writes are then complete.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                       Args&&... args) {
+cudaError_t launch_kernel(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -89,15 +93,16 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-#define ZSAA_LAUNCH(...)                          \
-  do {                                            \
-    cudaError_t le_ = ::zsaa::launch_pdl(__VA_ARGS__); \
-    if (le_ != cudaSuccess) return le_;           \
+#define ZSAA_LAUNCH_EARLY(early, ...)                                  \
+  do {                                                                 \
+    cudaError_t le_ = ::zsaa::launch_kernel(early, __VA_ARGS__);       \
+    if (le_ != cudaSuccess) return le_;                                \
   } while (0)
+#define ZSAA_LAUNCH(...) ZSAA_LAUNCH_EARLY(true, __VA_ARGS__)
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
   unsigned long long t;

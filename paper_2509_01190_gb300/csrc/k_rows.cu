@@ -755,7 +755,7 @@ cudaError_t launch_embed(int dtype, const void* E, const int32_t* tok, int rows,
                          int d, void* h, int32_t* pos, int* status, cudaStream_t s) {
   const int esz = dtype == ZSAA_BF16 ? 2 : 4;
   const int vec = d * esz / 16;
-  ZSAA_LAUNCH(embed_kernel, dim3(row_blocks(rows)), dim3(32 * kWarpsPerBlock), 0, s, 
+  ZSAA_LAUNCH_EARLY(false, embed_kernel, dim3(row_blocks(rows)), dim3(32 * kWarpsPerBlock), 0, s,
       static_cast<const uint4*>(E), tok, rows, L, vocab, vec, static_cast<uint4*>(h), pos, status);
   return cudaGetLastError();
 }
@@ -868,10 +868,11 @@ cudaError_t launch_rows_norm(int dtype, const void* src, const int32_t* tok, int
   return norm_dispatch(dtype, d, [&](auto t, int vec, auto q) -> cudaError_t {
     using T = decltype(t);
     constexpr int Q = decltype(q)::value;
-    ZSAA_LAUNCH(rows_norm_kernel<T, Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
-                static_cast<size_t>(vec) * 16, s, static_cast<const uint4*>(src), idx == nullptr ? tok : nullptr,
-                vocab, L, idx, N, k, pos_in, rows, vec, static_cast<const uint4*>(w), eps,
-                static_cast<uint4*>(h_out), static_cast<uint4*>(x_out), pos_out, status, cu_src, cu_dst, nseq);
+    ZSAA_LAUNCH_EARLY(idx != nullptr, rows_norm_kernel<T, Q>, dim3(norm_grid(rows, Q)), dim3(32 * kWarpsPerBlock),
+                      static_cast<size_t>(vec) * 16, s, static_cast<const uint4*>(src),
+                      idx == nullptr ? tok : nullptr, vocab, L, idx, N, k, pos_in, rows, vec,
+                      static_cast<const uint4*>(w), eps, static_cast<uint4*>(h_out), static_cast<uint4*>(x_out),
+                      pos_out, status, cu_src, cu_dst, nseq);
     return cudaGetLastError();
   });
 }

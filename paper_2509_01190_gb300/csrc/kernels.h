@@ -8,6 +8,9 @@
 namespace zsaa {
 
 // ---- row kernels (k_rows.cu)
+// The embedding (here and in launch_rows_norm) is the first kernel of a forward
+// or decode step and starts after everything before it on the stream has ended:
+// the kernels that follow read weights early.
 cudaError_t launch_embed(int dtype, const void* E, const int32_t* tok, int rows, int L, int vocab,
                          int d, void* h, int32_t* pos, int* status, cudaStream_t s);
 cudaError_t launch_rmsnorm(int dtype, const void* h, const void* w, int rows, int d, float eps,

@@ -196,3 +196,49 @@ def test_forward_host_pinned_streams_head(z, vocab):
         z.zsaa_forward_host(model, tok, B, L, 2.0, logits_h, kept_h)
         np.testing.assert_array_equal(logits_h.numpy(), res["nat_logits"])
         np.testing.assert_array_equal(kept_h.numpy(), res["kept_nat"])
+
+
+# A forward or decode step directly after a library call that writes one of its
+# weights (the residual epilogue merging an update into wq) reads the new values:
+# bitwise what it computes when the stream is idle in between.
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_weights_written_just_before(z, dtype):
+    shape = dataclasses.replace(SMALL_BF16 if dtype == "bf16" else I.TINY_F32, n_layers=2, prune="1")
+    code = z.ZSAA_BF16 if dtype == "bf16" else z.ZSAA_F32
+    B, L, K, d = 1, 40, 4096, shape.d_model
+    tok = torch.from_numpy(I.make_tokens(B, L, shape.vocab)).cuda()
+    up = torch.randn(2, d, K, device="cuda", generator=torch.Generator("cuda").manual_seed(3)) * 0.05
+    up = up.to(I.torch_dtype(shape))
+    got = {}
+    for idle in (True, False):
+        w = I.make_weights(shape, device="cuda")
+        model = z.Model(z.config_from_shape(shape), w, B, L)
+        z.zsaa_model_set_graphs(model, False)
+        sched, _ = z.zsaa_plan(model, L, 1.5)
+        outs = []
+
+        def merge():
+            wq = w["layers"][0]["wq"]
+            torch.cuda.synchronize()
+            z.zsaa_op_linear(up[0], up[1], None, wq, wq, d, d, K, code, z.EPI_RESID)
+            if idle:
+                torch.cuda.synchronize()
+
+        for _ in range(5):
+            outs.append(torch.empty(B, sched[-1], shape.vocab, device="cuda"))
+            merge()
+            z.zsaa_forward(model, tok, B, L, 1.5, outs[-1])
+        if dtype == "bf16":
+            cache = z.Cache(model, B, L, 1.5, 3)
+            pre = torch.empty(B, shape.vocab, device="cuda")
+            z.zsaa_prefill(model, cache, tok, pre)
+            for step in range(3):
+                outs.append(torch.empty(B, shape.vocab, device="cuda"))
+                step_tok = tok[:, step].contiguous()
+                merge()
+                z.zsaa_decode_step(model, cache, step_tok, outs[-1])
+        z.zsaa_sync(model)
+        got[idle] = outs
+    for a, b in zip(got[True], got[False]):
+        assert torch.equal(a, b)
+    assert not torch.equal(got[True][0], got[True][1])  # the update shows
