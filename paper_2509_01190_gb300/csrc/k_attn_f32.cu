@@ -18,6 +18,8 @@
 // heads of 64, 81-384 rows); the tiles take 35 and 31 us.
 // R is the largest of 8, 4, 2 that still gives two CTAs per SM: short
 // sequences take smaller tiles instead of leaving most SMs idle.
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -162,8 +164,8 @@ __global__ void __launch_bounds__(AF_THREADS)
     }
     cp_async_wait<1>();
     __syncthreads();  // V of this block has landed (and this block's P rows are written)
-#pragma unroll 2
-    for (int k = 0; k < AF_COLS; k += 4) {
+    // O += P V of keys k..k+3, of row i the first vis + 8 i keys of the block
+    auto add4 = [&](int k, int vis, auto edge) {
       uint64_t v[4][NP];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -181,14 +183,25 @@ __global__ void __launch_bounds__(AF_THREADS)
       }
 #pragma unroll
       for (int i = 0; i < R; ++i) {
+        if (edge && k >= vis + 8 * i) continue;
         const float4 p4 = *reinterpret_cast<const float4*>(sP + (ty + 8 * i) * AF_PLD + k);
         const uint64_t p2[4] = {f2pack(p4.x, p4.x), f2pack(p4.y, p4.y), f2pack(p4.z, p4.z), f2pack(p4.w, p4.w)};
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
+        for (int e = 0; e < 4; ++e) {
+          if (edge && k + e >= vis + 8 * i) continue;
 #pragma unroll
           for (int c = 0; c < NP; ++c) o[i][c] = ffma2(p2[e], v[e][c], o[i][c]);
+        }
       }
-    }
+    };
+    // keys that every row sees (V past the sequence's end is zero), then those on
+    // the diagonal: a hidden key's P is 0, but its V need not be finite, so its
+    // products are left out
+    const int all = causal ? max(0, min(AF_COLS, q0 + 1 - k0)) & ~3 : AF_COLS;
+#pragma unroll 2
+    for (int k = 0; k < all; k += 4) add4(k, 0, std::false_type());
+#pragma unroll 2
+    for (int k = all; k < min(AF_COLS, q0 + BQ - k0); k += 4) add4(k, q0 + ty + 1 - k0, std::true_type());
     __syncthreads();  // every thread is done with V and P
     if (kb + 1 < n_kb) af_load<HD>(sV, Vg, ld, k0 + AF_COLS, AF_COLS, N);
     cp_async_commit();

@@ -77,3 +77,28 @@ def test_forward_f32_head_sizes(z, d, heads, kv, hd, L):
     shape = dataclasses.replace(I.TINY_F32, name="f32-heads", d_model=d, n_heads=heads, n_kv_heads=kv, head_dim=hd,
                                 ffn_dim=200, vocab=333)
     check_case(run_case(z, shape, 2, L, 2.0, seqs=[0, 1]), "f32")
+
+
+# Causal rows do not see later keys, whatever those hold: with a key and value of
+# NaN or infinity the rows before are bitwise unchanged (tiles of 64, 32 and 16 rows,
+# the poisoned row first, inside and last in its 64-key block).
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("B,N,Hq,Hkv,hd", [(4, 257, 32, 8, 64), (2, 257, 12, 4, 32), (1, 130, 2, 1, 128),
+                                           (4, 193, 40, 8, 128), (1, 70, 3, 3, 64), (1, 70, 2, 1, 96)])
+def test_attention_f32_hides_later_rows(z, B, N, Hq, Hkv, hd, bad):
+    qkv = _qkv(B, N, Hq, Hkv, hd, 17, torch.float32)
+
+    def run(x):
+        out = torch.empty(B, N, Hq * hd, device="cuda")
+        lse = torch.empty(B, Hq, N, device="cuda")
+        z.zsaa_op_attention_ex(x, B, N, Hq, Hkv, hd, z.ZSAA_F32, True, out, lse)
+        torch.cuda.synchronize()
+        return out, lse
+
+    want, want_lse = run(qkv)
+    for j in (5, 31, 64, N - 1):
+        x = qkv.clone()
+        x.view(B, N, -1)[:, j, Hq * hd:] = bad
+        got, lse = run(x)
+        assert torch.equal(got[:, :j], want[:, :j]) and torch.equal(lse[:, :, :j], want_lse[:, :, :j]), j
+        assert not torch.isfinite(got[:, j]).any()
