@@ -1070,20 +1070,21 @@ bool bn_ok(int BN, int epi, const TcWeights& W, const GemmParams& p) {
 // So the split pays only on deep K (8B down: 1536 rows 145.5 -> 114.3 us,
 // 5084 rows 397.2 -> 364.2 us); on 64 k-blocks it measured 3-37% slower.
 struct TailPlan {
-  int S;  // k-parts per remainder tile; 1: whole tiles only
+  int S;      // k-parts per remainder tile; 1: whole tiles only
+  double us;  // modelled time of the whole plan
 };
 TailPlan tail_plan(int total, int units, int kb, double step_us, bool can_split, int max_slots) {
   const int W = total / units, R = total - W * units;
-  TailPlan tp{1};
-  if (!can_split || R == 0 || kb < kDeepKb) return tp;
   const double tw = kb * step_us;
-  double best = tw * std::min(1.0, 0.25 + 4.0 * R / units);
+  double best = R == 0 ? 0.0 : tw * std::min(1.0, 0.25 + 4.0 * R / units);
+  TailPlan tp{1, W * tw + best};
+  if (!can_split || R == 0 || kb < kDeepKb) return tp;
   for (int S = 2; S <= 8; ++S) {
     if (kb / S < 8 || R * (S - 1) > max_slots || R * S > units) break;
     const double t = tw / S + 8.0 + 5.5 * (S - 1);
     if (t < best - 1e-9) {
       best = t;
-      tp.S = S;
+      tp = TailPlan{S, W * tw + t};
     }
   }
   return tp;
@@ -1107,9 +1108,9 @@ int apply_tail(TileSched& t, int units, const TailPlan& tp) {
 }
 
 // Very deep K and more than two 128-row tiles: whether every 256 x 256 pair tile
-// can be cut into two k-parts that run in one round.  8B down (N 4096, 224
-// k-blocks), 257..512 rows: 47-48 us, against 68 for one wave of whole 128-wide
-// tiles.
+// can be cut into two k-parts that run in one round (taken where the model finds
+// that faster than the one-CTA plan).  8B down (N 4096, 224 k-blocks), 257..512
+// rows: 47-48 us, against 68 for one wave of whole 128-wide tiles.
 bool pair_parts_fit(int epi, int M, int N, int num_kb, int slots, int cta_slots) {
   const int tiles = ((M + 255) / 256) * ((N + P_BN - 1) / P_BN);
   return epi != kEpiSwiGLU && num_kb >= kVeryDeepKb && M > 2 * BM && 2 * slots <= kMaxGemmCtas &&
@@ -1140,6 +1141,7 @@ struct TilePlanIn {
 struct TilePlanOut {
   int BN, grid;
   TileSched ts;
+  bool parts;  // the pairs run every tile in k-parts (pair_parts_fit)
   int pairs;
   TileSched ps;
 };
@@ -1152,8 +1154,8 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
   const int m_tiles = (in.M + BM - 1) / BM;
   const int num_kb = in.K / BK;
   int BN = 0;
-  bool plan_pairs = false;
-  TailPlan plan_tp{1};
+  bool plan_pairs = false, plan_parts = false;
+  TailPlan plan_tp{1, 0.0};
   if (num_kb >= kDeepKb) {
     // Deep K (>= 64 k-blocks: every 8B projection, the 1B down projection):
     // the plan with the least waves x cost of one k-block step
@@ -1186,9 +1188,20 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
     if (slots > 0 && m_tiles >= 2) {
       const int ptiles = ((m_tiles + 1) / 2) * ((vn + P_BN - 1) / P_BN);
       const double cost = static_cast<double>((ptiles + slots - 1) / slots) * 0.34;
-      // (pair tiles that all fit one round in two k-parts: half a wave and the
-      // hand-off, which whole narrow tiles cannot reach)
-      if (cost < best - 1e-9 || pair_parts_fit(epi, in.M, in.N, num_kb, slots, can_split ? cta_slots : 0)) {
+      // Pair tiles that all fit one round in k-parts, against the one-CTA tiles and
+      // their own parts: half a wave and the hand-off, which whole narrow tiles
+      // cannot reach, but their parts do where there are few.  (The model has the
+      // one-CTA parts about 5% too fast: N 1024, K 12288, 800 rows 39.4 us modelled
+      // against 40.8 for pairs, measured 34.9 and 32.5.  With the pairs wherever
+      // they fit, N 256 and 1100 rows took 58.6 us against 27.1, N 512 31.2 against 27.1.)
+      if (pair_parts_fit(epi, in.M, in.N, num_kb, slots, can_split ? cta_slots : 0)) {
+        const TailPlan pair = tail_plan(ptiles, slots, num_kb, 0.34, true, cta_slots / 2);
+        const bool one_split = can_split && sms <= kMaxGemmCtas;
+        plan_parts = pair.S > 1 &&
+                     (BN == 0 ||
+                      pair.us < 1.05 * tail_plan(best_tiles, sms, num_kb, step_us(BN), one_split, cta_slots).us);
+      }
+      if (cost < best - 1e-9 || plan_parts) {
         BN = P_BN;
         plan_pairs = true;
         best_tiles = ptiles;
@@ -1288,12 +1301,13 @@ bool plan_tiles(const TilePlanIn& in, TilePlanOut& o) {
         pairs = static_cast<int>(g < 1 ? 1 : (g < slots ? g : slots));
       }
     } else if (plan_pairs) {
-      pairs = apply_tail(ps, slots, TailPlan{1});
+      pairs = apply_tail(ps, slots, TailPlan{1, 0.0});
     } else if (num_kb < kDeepKb) {
       const int waves_one = (ts.total + sms - 1) / sms;
-      if (waves_pair * kPairTileCost < waves_one && waves_one >= 2) pairs = apply_tail(ps, slots, TailPlan{1});
+      if (waves_pair * kPairTileCost < waves_one && waves_one >= 2) pairs = apply_tail(ps, slots, TailPlan{1, 0.0});
     }
   }
+  o.parts = plan_parts;
   o.BN = BN;
   o.grid = grid;
   o.ts = ts;
@@ -1321,9 +1335,6 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const TcWeights& W, int epi,
   const int cta_slots = can_split ? static_cast<int>(std::min<size_t>(
                                         p.splitk_ws_elems / (static_cast<size_t>(BM) * 256), kSplitKFlags / 4))
                                   : 0;
-  const bool parts = p.M > 320 && p.N >= 4096 && pair_parts_fit(epi, p.M, p.N, p.K / BK, slots, cta_slots);
-  if (!parts && swap_preferred(epi, p.M, p.N, p.K) && swap_supported(A, lda, W, epi, p))
-    return launch_gemm_swap(A, lda, W, epi, p, s);
   const int vn = epi == kEpiSwiGLU ? 2 * p.N : p.N;
   TilePlanIn in;
   in.epi = epi;
@@ -1338,7 +1349,11 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const TcWeights& W, int epi,
   in.bn128 = bn_ok(128, epi, W, p);
   in.bn256 = bn_ok(256, epi, W, p);
   TilePlanOut pl;
-  if (!plan_tiles(in, pl)) return cudaErrorInvalidValue;
+  const bool planned = plan_tiles(in, pl);
+  const bool parts = planned && pl.parts && p.M > 320 && p.N >= 4096;
+  if (!parts && swap_preferred(epi, p.M, p.N, p.K) && swap_supported(A, lda, W, epi, p))
+    return launch_gemm_swap(A, lda, W, epi, p, s);
+  if (!planned) return cudaErrorInvalidValue;
   const int BN = pl.BN, grid = pl.grid, pairs = pl.pairs;
   TileSched ts = pl.ts, ps = pl.ps;
   ts.ws = ps.ws = p.splitk_ws;

@@ -145,6 +145,17 @@ def test_gb300_plans_of_known_shapes(zlib):
     assert all(i[4] == 0 for i in items)
 
 
+# Very deep K in one round: pair tiles in k-parts only where they beat the one-CTA
+# tiles and their own parts, never as whole tiles on a few SMs.
+@pytest.mark.parametrize("M,N,K,pairs,parts", [(1100, 256, 12288, 0, 3), (800, 512, 12288, 0, 3), (257, 16, 12288, 0, 1),
+                                               (640, 128, 14336, 0, 1), (800, 1024, 12288, 1, 3),
+                                               (1500, 1536, 12288, 1, 2), (336, 4096, 14336, 1, 2)])
+def test_very_deep_k_plans(zlib, M, N, K, pairs, parts):
+    for epi in (EPI["store"], EPI["resid"], EPI["f32"]):
+        plan, _ = check_schedule(zlib, epi, M, N, K)
+        assert (plan[1], plan[10]) == (pairs, parts), plan
+
+
 def test_random_shapes_and_devices(zlib):
     rng = np.random.default_rng(2509)
     for _ in range(400):
