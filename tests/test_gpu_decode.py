@@ -80,13 +80,14 @@ def run_generate(z, shape, B, L, T, accel, seed=42):
                 prefill_logits=lg0.cpu().numpy(), step_logits=np.stack([s.cpu().numpy() for s in steps], 1))
 
 
-def check_generate(z, shape, res, B, L, T):
+def check_generate(z, shape, res, B, L, T, step_sigma=0.0):
+    """step_sigma: std of a further, stated difference of the decode steps' logits."""
     ores = res["ores"]
     mx, mean = logits_report(res["prefill_logits"], ores["prefill"]["logits"][:, -1])
     assert mx <= BF16_MAX_ABS and mean <= BF16_MEAN_ABS, ("prefill", mx, mean)
     for t in range(T):
         mx, mean = logits_report(res["step_logits"][:, t], ores["logits"][:, t])
-        assert mx <= BF16_MAX_ABS and mean <= BF16_MEAN_ABS, ("step", t, mx, mean)
+        assert mx <= BF16_MAX_ABS + 5 * step_sigma and mean <= BF16_MEAN_ABS + 0.8 * step_sigma, ("step", t, mx, mean)
     Hkv, hd = shape.n_kv_heads, shape.head_dim
     for layer in range(1, shape.n_layers + 1):
         info, k, v, pos = cache_views(z, res["cache"], layer, B, Hkv, hd)
