@@ -19,6 +19,17 @@ def need_gpu():
         pytest.skip("needs a CUDA device")
 
 
+def planned_gemm(z, epi, M, N, K, hd=64):
+    """(plan, items) of zsaa_gemm_schedule for the device at hand, on which the
+    call then runs.  The library asks the device for its SMs and for the CTA
+    pairs that fit at once, half as many on a GB300; elsewhere the two could
+    differ, so the test is skipped."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms != 152:
+        pytest.skip("the plan is stated for 152 SMs and 76 CTA pairs, this device has %d SMs" % sms)
+    return z.zsaa_gemm_schedule(epi, M, N, K, hd, sms, sms // 2, 256)
+
+
 def oracle_cfg(shape, prune_layers=None, n_layers=None):
     return O.OracleConfig(
         n_layers=shape.n_layers if n_layers is None else n_layers, d_model=shape.d_model,

@@ -33,7 +33,8 @@ def _run(z, qkv, B, N, Hq, Hkv, hd, causal, out=None):
 
 
 # Odd ratios pair query blocks (an odd number of blocks leaves a tile empty);
-# lengths around the 16-key, 32-column and 128-row edges, many short items.
+# lengths around the 16-key, 32-column and 128-row edges, many short items.  (Up to
+# 64 rows these calls run the mma.sync kernel; see the next test.)
 @pytest.mark.parametrize("causal", [True, False])
 @pytest.mark.parametrize("B,N,Hq,Hkv,hd", [(2, 1, 1, 1, 64), (3, 15, 3, 1, 128), (2, 16, 2, 2, 64), (2, 17, 4, 1, 64),
                                            (1, 33, 5, 1, 64), (2, 64, 3, 3, 128), (1, 96, 2, 1, 64), (2, 111, 4, 1, 128),
@@ -49,6 +50,68 @@ def test_attention_tiles(z, B, N, Hq, Hkv, hd, causal):
     assert np.all(bf16_ulp_close(got, ref_b, 1, 1e-5 * np.abs(ref_o).max(axis=-1, keepdims=True)))
     assert np.mean(got == ref_b) > 0.95
     np.testing.assert_allclose(_np(lse), ref_lse, rtol=1e-5, atol=1e-4)
+
+
+# Sequences of up to 64 rows on the tcgen05 kernel, which packed batches with longer
+# ones in them give it: alone they reach it in batches past the mma.sync kernel's
+# grid (65535 sequences; heads of 128 dims: 512 heads in all).  Lengths around the
+# 16-key steps and 32-column chunks of the only key block, next to other sequences'
+# rows; a sample of the sequences against the oracle, all of them for being there.
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("N,Hq,Hkv,hd", [(1, 2, 1, 64), (15, 1, 1, 64), (16, 2, 1, 64), (17, 3, 1, 64), (33, 2, 2, 64),
+                                         (37, 2, 1, 64), (63, 1, 1, 64), (64, 2, 1, 64), (1, 3, 1, 128),
+                                         (17, 2, 1, 128), (37, 3, 1, 128), (48, 4, 1, 128), (64, 1, 1, 128)])
+def test_short_sequences_on_tcgen05(z, N, Hq, Hkv, hd, causal):
+    B = 65537 if hd == 64 else 513 // Hq + 1
+    qkv = torch.randn(B * N, (Hq + 2 * Hkv) * hd, device="cuda", dtype=torch.bfloat16,
+                      generator=torch.Generator("cuda").manual_seed(N))
+    out, lse = _run(z, qkv, B, N, Hq, Hkv, hd, causal)
+    assert torch.isfinite(out).all() and torch.isfinite(lse).all()
+    at = torch.tensor(sorted({*range(0, B, max(1, B // 24)), B - 2, B - 1}), device="cuda")
+    pick = lambda t: t.view(B, N, -1)[at].reshape(len(at) * N, -1)
+    ref_o, ref_lse, _, _ = _oracle_attention(pick(qkv), len(at), N, Hq, Hkv, hd, causal=causal)
+    got, ref_b = _np(pick(out)).reshape(ref_o.shape), O.bf16_round(ref_o)
+    # the bounds of test_attention_tiles
+    assert np.all(bf16_ulp_close(got, ref_b, 1, 1e-5 * np.abs(ref_o).max(axis=-1, keepdims=True)))
+    assert np.mean(got == ref_b) > 0.95
+    np.testing.assert_allclose(_np(lse[at]), ref_lse, rtol=1e-5, atol=1e-4)
+
+
+# A packed sequence whose token embeddings are not finite leaves the others as they
+# are, bit for bit, in attention, column mass, selection and compaction: packed
+# batches of the tcgen05 kernel (one long sequence) and of the mma.sync one (all
+# short), first key blocks that end off the 16-key steps.
+@pytest.mark.parametrize("lengths", [[37, 21, 300, 13, 150], [37, 21, 40, 13, 64]])
+@pytest.mark.parametrize("accel", [1.0, 2.0])
+def test_packed_sequences_ignore_each_other(z, lengths, accel):
+    for shape in (SMALL_BF16, SMALL_BF16_128):
+        w = I.make_weights(shape, device="cuda")
+        toks = torch.from_numpy(I.make_tokens(1, sum(lengths), shape.vocab - 2)[0]).cuda()
+        bad_rows = [1, 3]
+        at = [sum(lengths[:b]) for b in range(len(lengths) + 1)]
+        for b in bad_rows:  # NaN and infinity in the last two rows of the embedding
+            toks[at[b]:at[b + 1]] = shape.vocab - 2
+            toks[at[b] + 1:at[b + 1]:2] = shape.vocab - 1
+        model = z.Model(z.config_from_shape(shape), w, len(lengths), max(lengths))
+        sched, _ = z.zsaa_plan_varlen(model, lengths, accel)
+        n = [s[-1] for s in sched]
+        got = []
+        for bad in (False, True):
+            if bad:
+                w["embed"][-2], w["embed"][-1] = float("nan"), float("inf")
+                torch.cuda.synchronize()
+            logits = torch.empty(sum(n), shape.vocab, device="cuda")
+            kept = torch.empty(sum(n), device="cuda", dtype=torch.int32)
+            z.zsaa_forward_varlen(model, toks, lengths, accel, logits, kept)
+            z.zsaa_sync(model)
+            got.append((logits, kept))
+        off = 0
+        for b, nb in enumerate(n):
+            if b not in bad_rows:
+                assert torch.equal(got[0][1][off:off + nb], got[1][1][off:off + nb]), b
+                assert torch.equal(got[0][0][off:off + nb], got[1][0][off:off + nb]), b
+            off += nb
+        assert not torch.isfinite(got[1][0]).all()
 
 
 # Both sides of the lines between this kernel and the mma.sync one of short

@@ -10,7 +10,7 @@ import sys
 
 import pytest
 
-from tests.helpers import check_linear, linear_case, need_gpu
+from tests.helpers import check_linear, linear_case, need_gpu, planned_gemm
 
 pytestmark = pytest.mark.gpu
 
@@ -50,7 +50,8 @@ def test_one_cta_tiled_paths(zlib):
 @pytest.mark.parametrize("M,N,K", [(33, 9760, 4096), (129, 9808, 4096), (300, 14336, 4096)])
 def test_192_wide_swiglu_tiles(zlib, M, N, K):
     need_gpu()
-    plan, _ = zlib.zsaa_gemm_schedule(2, M, N, K, 64, 152, 76, 256)
+    # (N, K >= 4096: SwiGLU never takes the swapped kernel)
+    plan, _ = planned_gemm(zlib, 2, M, N, K)
     assert plan[0] == 192 and plan[1] == 0
     out, ref, tol = linear_case(zlib, "swiglu", M, N, K, 1450 + M)
     check_linear(out, ref, tol, "swiglu", f"M={M} N={N}")

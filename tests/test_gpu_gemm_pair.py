@@ -11,7 +11,7 @@ of the Llama-3.2-1B forward."""
 import pytest
 import torch
 
-from tests.helpers import check_linear, linear_case, need_gpu, rand_bf16
+from tests.helpers import check_linear, linear_case, need_gpu, planned_gemm, rand_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -64,12 +64,12 @@ def test_pair_large_1b_shapes(z, name, M, N, K):
 
 
 # Very deep K in one round of two k-parts per pair tile: the first row count that
-# leaves the swapped kernel (321), three 128-row tiles (the last pair half empty),
-# four, and ragged columns.
+# leaves the swapped kernel (321: such plans of more rows and N >= 4096 go ahead of
+# it), three 128-row tiles (the last pair half empty), four, and ragged columns.
 @pytest.mark.parametrize("epi", ["resid", "store"])
 @pytest.mark.parametrize("M,N,K", [(321, 4096, 12288), (384, 4112, 12288), (512, 4096, 14336)])
 def test_pair_two_parts_of_very_deep_k(z, epi, M, N, K):
-    plan, items = z.zsaa_gemm_schedule({"store": 0, "resid": 1}[epi], M, N, K, 64, 152, 76, 256)
+    plan, items = planned_gemm(z, {"store": 0, "resid": 1}[epi], M, N, K)
     assert plan[1] == 1 and {it[4] for it in items} == {1, 2}  # pairs; every tile in parts
     out, ref, tol = linear_case(z, epi, M, N, K, 950 + M)
     check_linear(out, ref, tol, epi, f"{epi} M={M}")

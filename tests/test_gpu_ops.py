@@ -267,9 +267,9 @@ def _oracle_attention(qkv, B, N, Hq, Hkv, hd, causal=True):
     return np.stack(outs), np.stack(lses), Ps, x
 
 
-# Shapes with an even number of query heads per KV head run the two-tile
-# kernel (k_attn_pp.cu) at every length, the short kept lengths of the deep
-# pruned layers included (18..255 keys); odd ratios pair query blocks.
+# Lengths above 64 run the two-tile kernel (k_attn_pp.cu: pairs of heads, or with an
+# odd ratio of query blocks), up to 64 the mma.sync kernel (k_attn.cu); the kept
+# lengths of the deep pruned layers (18..255 keys) are on both sides.
 @pytest.mark.parametrize("B,N,Hq,Hkv,hd", [(2, 1, 4, 2, 64), (2, 65, 4, 2, 64), (1, 200, 4, 1, 128),
                                            (2, 130, 8, 2, 128), (1, 64, 2, 2, 64), (2, 300, 4, 2, 64),
                                            (1, 517, 8, 2, 64), (1, 1024, 4, 4, 64), (2, 300, 4, 2, 128),
