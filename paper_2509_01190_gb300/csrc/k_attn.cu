@@ -491,8 +491,12 @@ __global__ void colmass_f32_kernel(const float* __restrict__ qkv, const float* _
 // 19.1; N = 64 and 64 sequences 28.7 / 19.9; N = 80 (two steps a row) 30.1 / 49.3.
 // Heads of 128: N = 64, 8 sequences of 32 heads 7.4 / 6.2, 19: 11.5 / 11.5, 64:
 // 33.1 / 37.9, so up to 512 heads in all.  With lengths that differ the mean
-// decides, up to twice that length (19 of 12..71: 18.2 / 12.5 with events).
-// (its grid holds 65535 sequences, its copies need aligned rows)
+// decides, up to twice that length (launches between events): 16 heads of 64
+// without groups 1.1-1.6x faster in every mix of 1..128 rows (19 sequences to 256);
+// 32 over 8: 19 of 12..71 16.3 / 14.2, 8 of 128 and 24 of 40 24.0 / 20.3, 16 of 127
+// and 16 of 1 23.6 / 24.0, but 128 of 96 and 128 of 30 110 / 139; 32 of 128 over 8
+// the same either way.
+// (Its grid holds 65535 sequences, its copies need aligned rows.)
 bool attention_short(const void* qkv, int hd, int B, int N, long long rows, int Hq) {
   return N <= 128 && rows <= 64LL * B && (hd == 64 || static_cast<long long>(B) * Hq <= 512) && B <= 65535 &&
          (reinterpret_cast<uintptr_t>(qkv) & 15) == 0;

@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(THREADS)
     // Short sequence, one candidate per thread: count the candidates ahead of
     // candidate j in (key descending, index ascending) order directly.  Rank <
     // need is the radix path's kept set (every key above the threshold, then
-    // equal keys lowest index first), without its four barrier-bound passes.
+    // equal keys lowest index first), with two barriers in all.
     uint32_t* skey = hist;  // THREADS keys; the padding (key 0) never counts
     const int j = tid;
     const uint32_t kj = j < n_cand ? order_key(s[j]) : 0u;

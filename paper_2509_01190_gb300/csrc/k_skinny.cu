@@ -31,7 +31,9 @@
 //    by 1/rms (a row's factor passes through the dot product), added up from the
 //    bands' sums in band order while the products run.  Rounding h * w to bf16
 //    where the norm kernel rounds h / rms * w is no less exact (and none at all
-//    where w is a power of two).
+//    where w is a power of two): a step's logits, 4 layers of the 1B shape, are
+//    off by 0.0096 either way with weights 1 + 0.3 randn (against 64 bits,
+//    relative; with norm kernels 0.0097), by 0.0082 with weights of 1 (0.0093).
 // The norm's weights are staged in shared memory before the wait: a step's
 // 1 GB of weights passes through L2 between their uses, so they come from HBM
 // (loaded after the wait they made this slower than the norm kernels, as did
