@@ -57,12 +57,12 @@ TRAFFIC = {
     # profiles/gemm_gate_up_swiglu_8b_traffic.md: the first layer's MLP at accel 4
     ("gemm_gate_up_swiglu", "8b"): {
         "launch": "gate/up + SwiGLU, M=7272 rows (layer 1 of the accel-4 forward), N=2x14336, K=4096",
-        "bytes": 1459261184.0,
+        "bytes": 1457405184.0,
         "algorithmic_bytes": 502956032.0,
         "sources": {
-            "paper_2509_01190_gb300/csrc/k_gemm_tc.cu": "1cc5bc8dcc12f35fcfff0c798d25d022dc3dc112f36021b32a3178cad8bccfec",
-            "paper_2509_01190_gb300/csrc/common.cuh": "e629752c9039f4ede210522a63499e7aa3f49e1eaf203b7643c2590eaba654b5",
-            "paper_2509_01190_gb300/csrc/kernels.h": "5e6507ad09323de35469e72df74d4cec67bb34e714139154f4168294bd30a729",
+            "paper_2509_01190_gb300/csrc/k_gemm_tc.cu": "3403ba2adfccd9814b61663261467af604344f2d75b55a04aa8053f76294f371",
+            "paper_2509_01190_gb300/csrc/common.cuh": "f84ed6e870202898c8c4c7000c0724b92f5237ad324a7cb6558f0cde2dcce369",
+            "paper_2509_01190_gb300/csrc/kernels.h": "d247225fde40545b6a85b3395a686cffa75788d3259f4872dfb943c26a709a90",
         },
     },
 }
